@@ -436,18 +436,16 @@ typedef struct {
  *  presolve constant), max |unscaled primal residual|, 0}.
  * Work is queued on `stream` (a cudaStream_t; NULL = legacy default) and the
  * call returns without waiting for it.
- * Scratch: a fixed array of 8192 x 8 doubles (512 KiB) in the library's
- * device image, held by every GPU that loads the library until exit.  LPs
- * with ceil(m/1024) + ceil(n/1024) > 8192 (about 8.4 million rows + columns)
- * are rejected with UC_EINVAL.  All calls share that array, so calls whose
- * device work overlaps (several streams or host threads at once) race and
- * must be serialised by the caller; no part of it needs to start at zero.
- * Set-up: every call looks up the array's device address for the current
- * device (cudaGetSymbolAddress, which allocates nothing), so a context that was
- * reset and re-created never gets a stale address, and makes sure the entry's
- * two kernels are loaded (cudaFuncGetAttributes).  Under CUDA's lazy module
- * loading the driver may take device memory for their code on the first call
- * on each device (and on the first call after a cudaDeviceReset); make that
+ * Scratch: a fixed array of 8192 x 8 doubles (512 KiB) and 8 KiB of counters in
+ * the library's device image, held by every GPU that loads the library until
+ * exit.  LPs with ceil(m/1024) + ceil(n/1024) > 8192 (about 8.4 million rows +
+ * columns) are rejected with UC_EINVAL.  All calls share that memory, so calls
+ * whose device work overlaps (several streams or host threads at once) race and
+ * must be serialised by the caller.
+ * Set-up: none; the kernel addresses its scratch itself, so a context that was
+ * reset and re-created never gets a stale address.  Under CUDA's lazy module
+ * loading the driver may take device memory for the kernel's code on the first
+ * call on each device (and on the first call after a cudaDeviceReset); make that
  * first call before starting any stream capture.  No cudaMalloc, cudaFree or
  * other allocating call is made. */
 int uc_kkt_noalloc(const uc_device_lp *lp, const double *x, const double *y, double omega, double *out,

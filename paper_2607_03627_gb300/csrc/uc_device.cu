@@ -26,6 +26,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <climits>
 #include <cmath>
@@ -940,28 +941,6 @@ __global__ void k_lane_copy(double *__restrict__ dst, const double *__restrict__
 // evaluation: per-CTA FP64 partials of both candidates (fixed reduction order)
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ bool slot_is_max(int s) { return (s % kSlots) == RPU || (s % kSlots) == RDU; }
-
-__device__ __forceinline__ void block_reduce_store(double (&acc)[kPart], double *out) {
-    __shared__ double sh[kThreads / 32][kPart];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int s = 0; s < kPart; s++) {
-        double v = acc[s];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            double w = __shfl_down_sync(0xffffffffu, v, o);
-            v = slot_is_max(s) ? nnmax(v, w) : v + w;
-        }
-        if (lane == 0) sh[warp][s] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < kPart) {
-        const int s = threadIdx.x;
-        double v = sh[0][s];
-        for (int w = 1; w < kThreads / 32; w++) v = slot_is_max(s) ? nnmax(v, sh[w][s]) : v + sh[w][s];
-        out[s] = v;
-    }
-}
 
 // Block reduction of an evaluation record with few FP64 instructions.  The 14
 // sum slots go through a transposed warp reduction: at each of five exchange
@@ -3117,88 +3096,234 @@ static int max_replays(const uc_session &X) { return X.o.max_iter / X.o.n_eval +
 // 512 KiB) until the process exits.
 // ---------------------------------------------------------------------------
 constexpr int kNoAllocSlots = 8;         // Slot entries RP2 .. BND (DY2 stays 0)
-constexpr int kNoAllocRows = 1024;       // rows or columns per CTA of the allocation-free evaluation
-constexpr int kNoAllocMaxBlocks = 8192;  // CTAs of 1024 rows or columns: n/1024 + m/1024 <= 8192
+constexpr int kNoAllocMaxBlocks = 8192;  // CTA records in the scratch
+// Rows or columns per CTA: 256 (one per thread) while all CTAs are resident at
+// once (four per SM), else 512 so, else 1024, which spreads a CTA's sums and its
+// division over four rows per thread.  Measured: 47 k rows + columns 14.6 us at
+// 256 (15.4 at 512), 227 k 20.9 us at 512 (27.4 at 256), 1.9 M 87.6 us at 1024
+// (96.2 at 512).  The size limit is that of 1024: n/1024 + m/1024 <= 8192.
+constexpr int kNoAllocRows = 1024;
+constexpr int kNoAllocSmall = 256;
+constexpr int kNoAllocCtas = 4;          // per SM (64 registers; 3 and 5 measured 5-7 % slower)
+constexpr int kNoAllocGroup = 64;        // CTAs whose records the last of them to end adds up
+constexpr int kNoAllocTickets = 16;      // counter sets, taken in turn by the calls
 
 static __device__ __align__(256) double g_kkt_scratch[kNoAllocMaxBlocks * kNoAllocSlots];
+// CTAs ended per group and groups ended; every counter wraps to zero with its
+// last arrival.  A set per call in turn: calls that overlap against the contract
+// spoil their own results (the scratch) but not the counts of later calls.
+static __device__ unsigned g_kkt_ended[kNoAllocTickets][kNoAllocMaxBlocks / kNoAllocGroup + 1];
 
-// CTA b < nbr: rows [1024 b, ...); else columns.  Same per-thread order and
-// block reduction as k_eval, current point only.
-__global__ void __launch_bounds__(kThreads) k_kkt_partials_noalloc(uc_device_lp lp, int nbr, const double *__restrict__ x,
-                                                                   const double *__restrict__ y, double *__restrict__ scratch) {
-    double acc[kPart];
+// row . v, entries in order, the loads of four entries in flight together; an
+// FMA step issues only if some lane needs it
+__device__ __forceinline__ double csr_dot(const int32_t *__restrict__ ci, const double *__restrict__ av,
+                                          const double *__restrict__ v, int k0, int k1) {
+    double s = 0.0;
+    const unsigned lanes = __activemask();
+#pragma unroll 1
+    while (__any_sync(lanes, k0 < k1)) {
+        int c[4];
+        double a[4], g[4];
 #pragma unroll
-    for (int s = 0; s < kPart; s++) acc[s] = 0.0;
-    const bool rows = (int)blockIdx.x < nbr;
-    if (rows) {
-        const int b0 = blockIdx.x * kNoAllocRows, b1 = min(lp.m, b0 + kNoAllocRows);
-        for (int i = b0 + threadIdx.x; i < b1; i += kThreads) {
-            double ax = 0.0;
-            for (int k = lp.A_rowptr[i]; k < lp.A_rowptr[i + 1]; k++) ax += lp.A_val[k] * x[lp.A_colidx[k]];
-            const double qi = lp.q[i];
-            double r = ax - qi;
-            if (i >= lp.m_eq && r > 0.0) r = 0.0;   // min(r, 0) that keeps a NaN
-            acc[RP2] += r * r;
-            acc[RPU] = nnmax(acc[RPU], fabs(r) / lp.Dr[i]);   // a NaN wins, as in k_eval
-            acc[QY] += qi * y[i];
+        for (int q = 0; q < 4; q++)
+            if (k0 + q < k1) { c[q] = ld_stream(ci + k0 + q); a[q] = ld_stream(av + k0 + q); }
+#pragma unroll
+        for (int q = 0; q < 4; q++) if (k0 + q < k1) g[q] = __ldg(v + c[q]);
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            if (!__any_sync(lanes, k0 + q < k1)) break;
+            if (k0 + q < k1) s = fma(a[q], g[q], s);
         }
-    } else {
-        const int b0 = (blockIdx.x - nbr) * kNoAllocRows, b1 = min(lp.n, b0 + kNoAllocRows);
-        for (int j = b0 + threadIdx.x; j < b1; j += kThreads) {
-            double t = 0.0;
-            for (int k = lp.AT_rowptr[j]; k < lp.AT_rowptr[j + 1]; k++) t += lp.AT_val[k] * y[lp.AT_colidx[k]];
-            const double cj = lp.c[j], lj = lp.l[j], uj = lp.u[j];
-            const bool lf = isfinite(lj), uf = isfinite(uj);
-            const double lm = cj - t;
-            const double lpj = (lf && uf) ? lm : lf ? fmax(lm, 0.0) : uf ? fmin(lm, 0.0) : 0.0;
-            const double rd = lm - lpj;
-            double bnd = 0.0;
-            if (lf) bnd += lj * fmax(lpj, 0.0);
-            if (uf) bnd += uj * fmin(lpj, 0.0);
-            acc[RD2] += rd * rd;
-            acc[RDU] = nnmax(acc[RDU], fabs(rd) / lp.Dc[j]);
-            acc[CX] += cj * x[j];
-            acc[BND] += bnd;
-        }
+        k0 += 4;
     }
-    // every CTA overwrites its own record, so nothing in the scratch needs clearing
-    __shared__ double rec[kPart];
-    block_reduce_store(acc, rec);
-    __syncthreads();
-    if (threadIdx.x < kNoAllocSlots) scratch[(size_t)blockIdx.x * kNoAllocSlots + threadIdx.x] = rec[threadIdx.x];
+    return s;
 }
 
-// one CTA: fixed-order reduction of the partials (same order as k_control)
-__global__ void __launch_bounds__(kThreads) k_kkt_finish_noalloc(int nblocks, const double *__restrict__ scratch,
-                                                                 double q_inf, double c_inf, double omega,
-                                                                 double *__restrict__ out) {
-    __shared__ double red[kThreads][kNoAllocSlots];
-    double acc[kNoAllocSlots];
-#pragma unroll
-    for (int s = 0; s < kNoAllocSlots; s++) acc[s] = 0.0;
-    for (int blk = threadIdx.x; blk < nblocks; blk += kThreads) {
-#pragma unroll
-        for (int s = 0; s < kNoAllocSlots; s++) {
-            const double v = scratch[(size_t)blk * kNoAllocSlots + s];
-            acc[s] = (s == RPU || s == RDU) ? nnmax(acc[s], v) : acc[s] + v;
+// Tests on bit patterns: an FP64 comparison or conversion costs the FP64 pipe as
+// much as an FMA, and the kernel is bound by that pipe.
+__device__ __forceinline__ unsigned long long mag_bits(double v) { return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffULL; }
+__device__ __forceinline__ bool is_nan(double v) { return mag_bits(v) > 0x7ff0000000000000ULL; }
+// |v| cut to FP32 (relative error < 2^-23), or NaN outside [2^-100, 2^100)
+__device__ __forceinline__ float mag_float(double v) {
+    const unsigned hi = (unsigned)__double2hiint(v) & 0x7fffffffu, lo = (unsigned)__double2loint(v);
+    if (hi - ((1023u - 100u) << 20) >= (200u << 20)) return __int_as_float(0x7fc00000);
+    return __uint_as_float(((hi - ((1023u - 127u) << 20)) << 3) | (lo >> 29));
+}
+
+// The largest |r| / d, exactly, with few FP64 divisions (each a long FP64
+// sequence).  A thread keeps its row of the largest FP32 estimate; rows whose
+// estimate is within its error of that, or has none (zero rows aside), divide at
+// once; at the end the rows within the error of the CTA's largest estimate do.
+struct MaxQuotient {
+    double mx = 0.0, r = 0.0, d = 1.0;
+    float e = 0.0f;
+    __device__ __forceinline__ void add(double r2, double d2) {
+        if (mag_bits(r2) == 0 && !is_nan(d2) && mag_bits(d2) != 0) return;
+        float e2;
+        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(e2) : "f"(mag_float(d2)));
+        e2 *= mag_float(r2);
+        if (!(e2 < e * 0.99999f)) {
+            if (e2 > e * 1.00001f && e2 >= 0.0f && !is_neg(d2)) { r = r2; d = d2; e = e2; }
+            else mx = nnmax(mx, fabs(r2) / d2);
         }
     }
-#pragma unroll
-    for (int s = 0; s < kNoAllocSlots; s++) red[threadIdx.x][s] = acc[s];
-    __syncthreads();
-    for (int h = kThreads / 2; h > 0; h >>= 1) {
-        if (threadIdx.x < h)
-            for (int s = 0; s < kNoAllocSlots; s++) {
-                const double a = red[threadIdx.x][s], c = red[threadIdx.x + h][s];
-                red[threadIdx.x][s] = (s == RPU || s == RDU) ? nnmax(a, c) : a + c;
-            }
+    __device__ __forceinline__ double finish(int *best) {
+        const int top = __reduce_max_sync(0xffffffffu, __float_as_int(e));
+        if ((threadIdx.x & 31) == 0) atomicMax(best, top);
         __syncthreads();
+        if (e > 0.0f && e >= __int_as_float(*(volatile int *)best) * 0.99999f) mx = nnmax(mx, fabs(r) / d);
+        return mx;
     }
+};
+
+// Sums of three slots and the maximum of a fourth (non-negative values) over the
+// CTA, in a fixed order, to out[0 .. 4).  The sums share their shuffles: after
+// two exchanges a lane holds one slot's partial sum of four lanes.
+__device__ __forceinline__ void kkt_block_sum(double a0, double a1, double a2, double mx, double *out) {
+    __shared__ double sh[kThreads / 32][4];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // lanes with bit 4 set keep slots 1 and (none), the others 0 and 2
+    const bool up = lane & 16;
+    double k0 = up ? a1 : a0;
+    const double s0 = up ? a0 : a1;
+    k0 += __shfl_xor_sync(0xffffffffu, s0, 16);
+    double k2 = a2 + __shfl_xor_sync(0xffffffffu, a2, 16);
+    // lanes with bit 3 set keep slot 2, the others slot 0 or 1
+    const bool up2 = lane & 8;
+    double v = (up2 ? k2 : k0) + __shfl_xor_sync(0xffffffffu, up2 ? k0 : k2, 8);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mx = nnmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if (lane == 0) { sh[warp][0] = v; sh[warp][3] = mx; }
+    if (lane == 16) sh[warp][1] = v;
+    if (lane == 8) sh[warp][2] = v;
+    __syncthreads();
+    if (threadIdx.x < 4) {
+        double t = sh[0][threadIdx.x];
+        for (int w = 1; w < kThreads / 32; w++) t = threadIdx.x == 3 ? nnmax(t, sh[w][threadIdx.x]) : t + sh[w][threadIdx.x];
+        out[threadIdx.x] = t;
+    }
+    __syncthreads();
+}
+
+// records [0, n) of kNoAllocSlots values summed by warp 0 in a fixed order; every
+// lane gets the sums (lane l adds records l / 8, l / 8 + 4, ... of slot l % 8)
+__device__ __forceinline__ double kkt_sum_records(const double *rec, int n, int stride) {
+    const int slot = threadIdx.x % kNoAllocSlots;
+    const bool mx = slot == RPU || slot == RDU;
+    double v = 0.0;
+    for (int k0 = threadIdx.x / kNoAllocSlots; k0 < n; k0 += 16) {
+        double t[4];
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            t[q] = 0.0;
+            if (k0 + 4 * q < n) t[q] = __ldcg(rec + (size_t)(k0 + 4 * q) * stride + slot);
+        }
+#pragma unroll
+        for (int q = 0; q < 4; q++) v = mx ? nnmax(v, t[q]) : v + t[q];
+    }
+#pragma unroll
+    for (int o = kNoAllocSlots; o < 32; o <<= 1) {
+        const double w = __shfl_xor_sync(0xffffffffu, v, o);
+        v = mx ? nnmax(v, w) : v + w;
+    }
+    return v;
+}
+
+// CTA b < nbr: rows [per b, ...); else columns.  The last CTA of each group to end
+// adds the group's records, the last group's adds those and writes the result.
+// Bound by the FP64 pipe and by latency (6,049-bus LP: the pipe is busy 70 % of
+// 96 us before the last two changes): so one launch instead of two, four entries'
+// loads of a row in flight together, FP64 instructions only for the products and
+// sums (bit tests for every comparison, a vote skips a warp's terms that are exact
+// zeros) and about one division per CTA instead of one per row and column.
+// 6,049 buses: 150.9 -> 87.6 us, 30 buses: 26.6 -> 12.4 us per call.
+__global__ void __launch_bounds__(kThreads, kNoAllocCtas) k_kkt_noalloc(uc_device_lp lp, int nbr, int per, const double *__restrict__ x,
+                                                          const double *__restrict__ y, double omega, int ticket,
+                                                          double *__restrict__ out) {
+    __shared__ double rec[kNoAllocSlots], sum[4];
+    __shared__ int best;
+    __shared__ bool last;
+    if (threadIdx.x == 0) best = 0;
+    if (threadIdx.x < kNoAllocSlots) rec[threadIdx.x] = 0.0;
+    __syncthreads();
+    double a0 = 0.0, a1 = 0.0, a2 = 0.0;
+    MaxQuotient quot;
+    const bool rows = (int)blockIdx.x < nbr;
+    if (rows) {                    // |r|^2, q.y, largest unscaled residual
+        const int b0 = blockIdx.x * per, b1 = min(lp.m, b0 + per);
+        for (int i = b0 + threadIdx.x; i < b1; i += kThreads) {
+            const int k0 = __ldg(lp.A_rowptr + i), k1 = __ldg(lp.A_rowptr + i + 1);
+            const double qi = ld_stream(lp.q + i), d = ld_stream(lp.Dr + i), yi = __ldg(y + i);
+            double r = csr_dot(lp.A_colidx, lp.A_val, x, k0, k1) - qi;
+            if (i >= lp.m_eq && !is_neg(r) && !is_nan(r)) r = 0.0;   // min(r, 0) that keeps a NaN
+            a0 = fma(r, r, a0);
+            if (__any_sync(__activemask(), mag_bits(qi) != 0 || !is_fin(yi))) a1 = fma(qi, yi, a1);
+            quot.add(r, d);
+        }
+    } else {                       // |rd|^2, c.x, bound part, largest unscaled reduced-cost residual
+        const int b0 = ((int)blockIdx.x - nbr) * per, b1 = min(lp.n, b0 + per);
+        for (int j = b0 + threadIdx.x; j < b1; j += kThreads) {
+            const int k0 = __ldg(lp.AT_rowptr + j), k1 = __ldg(lp.AT_rowptr + j + 1);
+            const double cj = ld_stream(lp.c + j), lj = ld_stream(lp.l + j), uj = ld_stream(lp.u + j);
+            const double d = ld_stream(lp.Dc + j), xj = __ldg(x + j);
+            const double lm = cj - csr_dot(lp.AT_colidx, lp.AT_val, y, k0, k1);
+            const bool lf = is_fin(lj), uf = is_fin(uj);
+            // reduced cost inside the cone the bounds allow (lp_j) and the rest (rd = lm - lp_j)
+            double rd, lp_j = 0.0;
+            if (lf && uf) {
+                if (!is_nan(lm)) lp_j = lm;
+                rd = is_fin(lm) ? 0.0 : __longlong_as_double(0x7ff8000000000000LL);
+            } else if (is_nan(lm)) {
+                rd = lm;
+            } else {
+                lp_j = lf ? pos_part(lm) : uf ? neg_part(lm) : 0.0;
+                rd = lf ? neg_part(lm) : uf ? pos_part(lm) : lm;
+            }
+            const double bound = is_neg(lp_j) ? (uf ? uj : 0.0) : (lf ? lj : 0.0);
+            const unsigned lanes = __activemask();
+            if (__any_sync(lanes, mag_bits(rd) != 0)) a0 = fma(rd, rd, a0);
+            if (__any_sync(lanes, mag_bits(cj) != 0 || !is_fin(xj))) a1 = fma(cj, xj, a1);
+            if (__any_sync(lanes, mag_bits(bound) != 0 && mag_bits(lp_j) != 0)) a2 = fma(bound, lp_j, a2);
+            quot.add(rd, d);
+        }
+    }
+    kkt_block_sum(a0, a1, a2, quot.finish(&best), sum);
+    if (threadIdx.x == 0) {
+        rec[rows ? RP2 : RD2] = sum[0];
+        rec[rows ? QY : CX] = sum[1];
+        if (!rows) rec[BND] = sum[2];
+        rec[rows ? RPU : RDU] = sum[3];
+    }
+    __syncthreads();
+    const int group = (int)blockIdx.x / kNoAllocGroup, ngroups = ((int)gridDim.x + kNoAllocGroup - 1) / kNoAllocGroup;
+    double *mine = g_kkt_scratch + (size_t)group * kNoAllocGroup * kNoAllocSlots;   // the group's records, its sum over the first
+    if (threadIdx.x < kNoAllocSlots)
+        __stcg(mine + (size_t)(blockIdx.x % kNoAllocGroup) * kNoAllocSlots + threadIdx.x, rec[threadIdx.x]);
+    if (threadIdx.x >= 32) return;
+    const int in_group = min(kNoAllocGroup, (int)gridDim.x - group * kNoAllocGroup);
+    auto ended = [&](unsigned *count, int of) {   // warp 0: whether this arrival is the last of `of`
+        __threadfence();
+        __syncwarp();
+        if (threadIdx.x == 0) last = atomicInc(count, (unsigned)(of - 1)) == (unsigned)(of - 1);
+        __syncwarp();
+        __threadfence();
+        return (bool)*(volatile bool *)&last;
+    };
+    if (!ended(&g_kkt_ended[ticket][1 + group], in_group)) return;
+    const double t = kkt_sum_records(mine, in_group, kNoAllocSlots);
+    __syncwarp();
+    if (threadIdx.x < kNoAllocSlots) __stcg(mine + threadIdx.x, t);
+    if (!ended(&g_kkt_ended[ticket][0], ngroups)) return;
+    const double v = kkt_sum_records(g_kkt_scratch, ngroups, kNoAllocGroup * kNoAllocSlots);
+    double T[kNoAllocSlots];
+#pragma unroll
+    for (int s = 0; s < kNoAllocSlots; s++) T[s] = __shfl_sync(0xffffffffu, v, s);
     if (threadIdx.x != 0) return;
-    const double *T = red[0];
     const double pobj = T[CX], dobj = T[QY] + T[BND], gap = pobj - dobj;
-    out[0] = T[RPU] / (1.0 + q_inf);
-    out[1] = T[RDU] / (1.0 + c_inf);
+    out[0] = T[RPU] / (1.0 + lp.q_inf);
+    out[1] = T[RDU] / (1.0 + lp.c_inf);
     out[2] = fabs(gap) / (1.0 + fabs(pobj) + fabs(dobj));
     out[3] = kkt_w(T[RP2], T[RD2], gap, omega);
     out[4] = pobj;
@@ -3206,33 +3331,6 @@ __global__ void __launch_bounds__(kThreads) k_kkt_finish_noalloc(int nblocks, co
     out[6] = T[RPU];
     out[7] = 0.0;
 }
-
-// Device address of g_kkt_scratch for the current device.  Looked up on every
-// call (cudaGetSymbolAddress allocates nothing), so a context that was reset
-// and re-created, where the array may sit elsewhere, never gets a stale
-// address.  The entry's kernels are loaded here too: under lazy module loading
-// the driver may take device memory for their code on first use, and this
-// moves that to the first call on a device.
-static int kkt_scratch_address(double **out) {
-    int dev = 0;
-    UC_CUDA(cudaGetDevice(&dev));
-    void *p = nullptr;
-    cudaError_t e = cudaGetSymbolAddress(&p, g_kkt_scratch);
-    if (e != cudaSuccess || !p) {
-        set_error("cudaGetSymbolAddress(scratch) failed on device %d: %s", dev, cudaGetErrorString(e));
-        return UC_ECUDA;
-    }
-    cudaFuncAttributes fa;
-    e = cudaFuncGetAttributes(&fa, k_kkt_partials_noalloc);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_kkt_finish_noalloc);
-    if (e != cudaSuccess) {
-        set_error("loading the KKT kernels failed on device %d: %s", dev, cudaGetErrorString(e));
-        return UC_ECUDA;
-    }
-    *out = (double *)p;
-    return UC_OK;
-}
-
 
 // ---------------------------------------------------------------------------
 // ||A||_2 for presolve on the device: power iteration on A^T A
@@ -3521,13 +3619,21 @@ int uc_kkt_noalloc(const uc_device_lp *lp, const double *x, const double *y, dou
                   "(n + m up to about 8.4 million)", (long long)(nbr64 + nbc64), dev::kNoAllocMaxBlocks);
         return UC_EINVAL;
     }
-    const int nbr = (int)nbr64, nblocks = (int)(nbr64 + nbc64);
-    double *scratch = nullptr;
-    int rc = dev::kkt_scratch_address(&scratch);
-    if (rc) return rc;
-    cudaStream_t s = (cudaStream_t)stream;
-    if (nblocks > 0) dev::k_kkt_partials_noalloc<<<nblocks, dev::kThreads, 0, s>>>(*lp, nbr, x, y, scratch);
-    dev::k_kkt_finish_noalloc<<<1, dev::kThreads, 0, s>>>(nblocks, scratch, lp->q_inf, lp->c_inf, omega, out);
+    int sms = 0, dev_id = 0;
+    UC_CUDA(cudaGetDevice(&dev_id));
+    UC_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev_id));
+    int per = dev::kNoAllocSmall;
+    int64_t nbr, nbc;
+    for (;; per *= 2) {
+        nbr = ((int64_t)lp->m + per - 1) / per;
+        nbc = ((int64_t)lp->n + per - 1) / per;
+        if (per == dev::kNoAllocRows || nbr + nbc <= (int64_t)dev::kNoAllocCtas * sms) break;
+    }
+    static std::atomic<unsigned> calls{0};
+    const int ticket = (int)(calls.fetch_add(1, std::memory_order_relaxed) % dev::kNoAllocTickets);
+    // an LP without rows and columns still writes its result
+    const int blocks = (int)std::max<int64_t>(1, nbr + nbc);
+    dev::k_kkt_noalloc<<<blocks, dev::kThreads, 0, (cudaStream_t)stream>>>(*lp, (int)nbr, per, x, y, omega, ticket, out);
     UC_CUDA(cudaGetLastError());
     return UC_OK;
 }
