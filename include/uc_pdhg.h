@@ -120,7 +120,9 @@ typedef struct {
     int n_eval;                  /* iterations between KKT / restart evaluations (default 64, even) */
     int use_graph;               /* 1: replay CUDA graphs of n_eval iterations (default 1) */
     int kernel_timing;           /* 1: time the primal and dual kernel of the middle iteration of every
-                                    replay with events (graph path only) */
+                                    replay with events (graph path only).  Where the resident kernel
+                                    runs all iterations (see spmv_kernel), its middle iteration is timed
+                                    on the device and split by the halves' FP64 instructions */
     double timeout_ms;           /* 0: none */
     const double *warm_x;        /* nullable [n] presolved-space primal start (scaled) */
     const double *warm_y;        /* nullable [m] presolved-space dual start (scaled) */
@@ -138,7 +140,11 @@ typedef struct {
                                     2 staged: persistent CTAs that copy each 128-row chunk's matrix
                                     rows and vectors into shared memory ahead of use (Halpern only,
                                     rows of at most 640 entries, else UC_EINVAL).  The strided slots
-                                    are not used by shared-matrix (lanes) sessions.  All variants give
+                                    are not used by shared-matrix (lanes) sessions.  With 0 and the
+                                    Halpern algorithm, a session (of up to 64 LPs) whose matrix and
+                                    vectors fit into the SMs' shared memory runs all iterations between
+                                    two evaluations in one cooperative launch instead; cta_rows,
+                                    rows_per_thread and no_pdl do not apply to it.  All variants give
                                     identical iterates. */
     int cta_rows;                /* threads per CTA of the iteration kernels: 0 (default 128), 128,
                                     256 or 512; results do not depend on it (tuning knob) */

@@ -19,7 +19,8 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 HOST_SOURCES = ["uc_host.cpp", "uc_crossover.cpp"]
 DEVICE_SOURCES = ["uc_device.cu"]
-HEADERS = [os.path.join(CSRC, "uc_internal.h"), os.path.join(INCLUDE, "uc_pdhg.h")]
+HEADERS = [os.path.join(CSRC, "uc_internal.h"), os.path.join(CSRC, "uc_block.cuh"),
+           os.path.join(INCLUDE, "uc_pdhg.h")]
 
 
 def _nvcc() -> str:

@@ -43,7 +43,11 @@ namespace uc {
 namespace dev {
 
 constexpr int kThreads = 256;      // threads per CTA of the row kernels (8 warps)
-constexpr int kEvalRows = 1024;    // rows handled by one CTA of the evaluation kernel
+// Rows handled by one CTA of the evaluation kernel, by the LP's rows + columns
+// (not the session's: a batch evaluates each LP as its single solve does).  Small
+// LPs take one per thread, so that the evaluation, which the FP64 pipe of the few
+// SMs it runs on bounds, spreads over four times the SMs.
+static int eval_rows(int64_t nm) { return nm <= 256 * 608 ? 256 : nm <= 512 * 608 ? 512 : 1024; }
 constexpr int kSlots = 9;          // reduction slots per candidate
 constexpr int kPart = 2 * kSlots;  // per-block partial record (current, average)
 
@@ -124,6 +128,8 @@ struct Bufs {
     // state: x, y double-buffered
     double *x[2], *y[2];
     double *xsum, *ysum, *xa, *ya, *xret, *yret;   // Halpern: xsum holds x-bar, xret/yret the map output
+    unsigned *blk_seq;                         // resident block kernel: iterations of all its launches so far
+    int n_eval;
     double *part;                              // per-CTA evaluation records
     double *red;                               // [k][kPart] reduced evaluation records
     Scalars *S;
@@ -748,6 +754,14 @@ __global__ void __launch_bounds__(kStRows, 8) k_iter_staged(const Chunk *__restr
     }
 }
 
+}  // namespace dev
+}  // namespace uc
+
+#include "uc_block.cuh"
+
+namespace uc {
+namespace dev {
+
 // ---------------------------------------------------------------------------
 // shared-matrix ("lanes") iteration kernels (Halpern): K = 2 or 4 LPs with one
 // scaled matrix, stored once; their vectors are interleaved, element j of lane
@@ -1013,6 +1027,34 @@ __device__ __forceinline__ bool is_fin(double v) {
 __device__ __forceinline__ double pos_part(double v) { return is_neg(v) ? 0.0 : v; }
 __device__ __forceinline__ double neg_part(double v) { return is_neg(v) ? v : 0.0; }
 
+// Terms that are exact zeros for a whole warp are skipped (the kernel is bound by
+// the FP64 pipe): any_bits: some value is not a zero; differ: a - b is not an
+// exact zero (two equal values that are not finite differ: inf - inf).
+__device__ __forceinline__ bool any_bits(unsigned lanes, double v) { return __any_sync(lanes, (__double_as_longlong(v) << 1) != 0); }
+__device__ __forceinline__ bool differ(double a, double b) { return __double_as_longlong(a) != __double_as_longlong(b) || !is_fin(a); }
+
+// f(value, g[j], j) for entries k0, k0 + step, ... < k1 of a row, in order; the
+// loads of four entries are in flight together (one after another they are the
+// evaluation's time: 6 round trips to L2 for a row of three entries instead of 3)
+template <typename VT, typename At, typename F>
+__device__ __forceinline__ void each_entry(const int *__restrict__ ci, const VT *__restrict__ v, const double *g, At at,
+                                           int k0, int k1, int step, F f) {
+    for (int k = k0; k < k1; k += 4 * step) {
+        size_t j[4];
+        double a[4], gj[4];
+#pragma unroll
+        for (int q = 0; q < 4; q++)
+            if (k + q * step < k1) { j[q] = at(__ldg(ci + k + q * step)); a[q] = widen(__ldg(v + k + q * step)); }
+#pragma unroll
+        for (int q = 0; q < 4; q++) if (k + q * step < k1) gj[q] = g[j[q]];
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            if (k + q * step >= k1) break;
+            f(a[q], gj[q], j[q]);
+        }
+    }
+}
+
 // mode 0: the start point (candidate 0 only); mode 1: regular evaluation.
 // Average variant: candidate 0 = current point, candidate 1 = average since the
 // last restart.  Halpern variant: candidate 0 = the last map output
@@ -1021,9 +1063,11 @@ __device__ __forceinline__ double neg_part(double v) { return is_neg(v) ? v : 0.
 // x_in / y_in being the input of the last step (buffer 1, n_eval even).
 // K > 1: shared-matrix session, vectors interleaved by lane; lane blockIdx.y.
 template <typename VT, int K>
-__global__ void __launch_bounds__(kThreads) k_eval(const Seg *__restrict__ segs, Bufs b, int mode) {
+__global__ void __launch_bounds__(kThreads, 3) k_eval(const Seg *__restrict__ segs, Bufs b, int mode) {
     const Seg sg = segs[blockIdx.x];
     const int lane = (K == 1) ? 0 : (int)blockIdx.y;
+    // a resident block kernel before this one has ended: the next one's tags differ from its tags
+    if (mode == 1 && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *b.blk_seq += (unsigned)b.n_eval;
     const Scalars *S = b.S + ((K == 1) ? sg.inst : lane);
     auto at = [lane](int idx) { return (size_t)idx * K + lane; };
     double acc[kPart];
@@ -1060,23 +1104,24 @@ __global__ void __launch_bounds__(kThreads) k_eval(const Seg *__restrict__ segs,
             const VT *__restrict__ v = static_cast<const VT *>(b.A_v);
             for (int i = sg.begin + threadIdx.x; i < sg.end; i += kThreads) {
                 double ax0 = 0.0, ax1 = 0.0, axin = 0.0;
-                for (int k = b.A_rp[i]; k < b.A_rp[i + 1]; k++) {
-                    const size_t j = at(b.A_ci[k]);
-                    const double a = widen(v[k]);
-                    ax0 += a * x[j];
-                    if (avg) ax1 += a * (xav[j] * inv_j);
-                    if (fprp) axin += a * b.x[1][j];
-                }
+                each_entry(b.A_ci, v, x, at, __ldg(b.A_rp + i), __ldg(b.A_rp + i + 1), 1, [&](double a, double xj, size_t j) {
+                    ax0 = fma(a, xj, ax0);
+                    if (avg) ax1 = fma(a, xav[j] * inv_j, ax1);
+                    if (fprp) axin = fma(a, b.x[1][j], axin);
+                });
                 const size_t ii = at(i);
                 const double qi = b.q[ii], idr = b.inv_Dr[ii], yh = b.ya[ii];
                 const bool ineq = i >= eq_end;
                 double r0 = ax0 - qi;
                 if (ineq && !is_neg(r0)) r0 = 0.0;
                 const double y0 = y[ii];
-                acc[RP2] += r0 * r0;
-                acc[RPU] = nnmax(acc[RPU], fabs(r0) * idr);
-                acc[QY] += qi * y0;
-                acc[DY2] += (y0 - yh) * (y0 - yh);
+                const unsigned lanes = __activemask();
+                if (any_bits(lanes, r0)) {
+                    acc[RP2] = fma(r0, r0, acc[RP2]);
+                    acc[RPU] = nnmax(acc[RPU], fabs(r0) * idr);
+                }
+                if (__any_sync(lanes, (__double_as_longlong(qi) << 1) != 0 || !is_fin(y0))) acc[QY] = fma(qi, y0, acc[QY]);
+                if (__any_sync(lanes, differ(y0, yh))) acc[DY2] = fma(y0 - yh, y0 - yh, acc[DY2]);
                 if (avg) {
                     double r1 = ax1 - qi;
                     if (ineq && !is_neg(r1)) r1 = 0.0;
@@ -1106,13 +1151,11 @@ __global__ void __launch_bounds__(kThreads) k_eval(const Seg *__restrict__ segs,
                  j += lng ? sg.end - j : kThreads) {
                 double t0 = 0.0, t1 = 0.0, tr = 0.0;
                 const int e0 = b.AT_rp[j] + (lng ? wl : 0), e1 = b.AT_rp[j + 1], es = lng ? 32 : 1;
-                for (int k = e0; k < e1; k += es) {
-                    const size_t i = at(b.AT_ci[k]);
-                    const double a = widen(v[k]);
-                    t0 += a * y[i];
-                    if (avg) t1 += a * (yav[i] * inv_j);
-                    if (ray) tr += a * (y[i] - b.y[1][i]);
-                }
+                each_entry(b.AT_ci, v, y, at, e0, e1, es, [&](double a, double yi, size_t i) {
+                    t0 = fma(a, yi, t0);
+                    if (avg) t1 = fma(a, yav[i] * inv_j, t1);
+                    if (ray) tr = fma(a, yi - b.y[1][i], tr);
+                });
                 if (lng) {
 #pragma unroll
                     for (int o = 16; o > 0; o >>= 1) {
@@ -1132,16 +1175,17 @@ __global__ void __launch_bounds__(kThreads) k_eval(const Seg *__restrict__ segs,
                     if (cnd == 1 && !avg) break;
                     const double lm = lam[cnd];
                     const double lp = (lf && uf) ? lm : lf ? pos_part(lm) : uf ? neg_part(lm) : 0.0;
-                    const double rd = lm - lp;
-                    double bnd = 0.0;
-                    if (lf) bnd += lj * pos_part(lp);
-                    if (uf) bnd += uj * neg_part(lp);
+                    const unsigned lanes = __activemask();
                     double *a = acc + cnd * kSlots;
-                    a[RD2] += rd * rd;
-                    a[RDU] = nnmax(a[RDU], fabs(rd) * idc);
-                    a[CX] += cj * xs[cnd];
-                    a[BND] += bnd;
-                    a[DX2] += (xs[cnd] - xh) * (xs[cnd] - xh);
+                    if (__any_sync(lanes, differ(lm, lp))) {   // a boxed column has none
+                        const double rd = lm - lp;
+                        a[RD2] = fma(rd, rd, a[RD2]);
+                        a[RDU] = nnmax(a[RDU], fabs(rd) * idc);
+                    }
+                    if (__any_sync(lanes, (__double_as_longlong(cj) << 1) != 0 || !is_fin(xs[cnd]))) a[CX] = fma(cj, xs[cnd], a[CX]);
+                    const double bound = is_neg(lp) ? (uf ? uj : 0.0) : (lf ? lj : 0.0);
+                    if (any_bits(lanes, bound)) a[BND] = fma(bound, lp, a[BND]);
+                    if (__any_sync(lanes, differ(xs[cnd], xh))) a[DX2] = fma(xs[cnd] - xh, xs[cnd] - xh, a[DX2]);
                 }
                 if (fpr) {
                     const double d = b.x[1][jj] - x[jj];
@@ -1192,11 +1236,18 @@ __global__ void __launch_bounds__(kThreads) k_reduce(const InstRange *__restrict
 }
 
 // ---------------------------------------------------------------------------
-// scalar controller: one thread per LP
+// scalar controller: one warp per LP
 // ---------------------------------------------------------------------------
+// Every FP64 quotient, root, logarithm and exponential is a long chain of FP64
+// instructions, and one thread takes them one after another: 10 us of the 35 us
+// an evaluation takes on the 30-bus LP.  Here the lanes of a warp take those that
+// do not depend on one another side by side (one instruction stream), the
+// scalars are read by all lanes and written by the first.
 __device__ double kkt_w(double rp2, double rd2, double gap, double w) {
     return sqrt(w * w * rp2 + rd2 / (w * w) + gap * gap);
 }
+
+__device__ __forceinline__ double lane_val(double v, int lane) { return __shfl_sync(0xffffffffu, v, lane); }
 
 // Primal weight at a restart from the epoch's movement dx (primal), dy (dual).
 // The error e = ln(omega dx / dy) is zero when the weighted movements
@@ -1204,16 +1255,23 @@ __device__ double kkt_w(double rp2, double rd2, double gap, double w) {
 // omega: ln omega <- ln omega - (kp e + ki sum(e) + kd (e - e_prev)).  PDLP's
 // rule, omega <- exp(0.5 ln(dy/dx) + 0.5 ln omega), is the proportional part
 // with kp = 0.5 and is computed in that form.  omega is kept when dx or dy is
-// at most 1e-10.
-__device__ double primal_weight(Scalars *S, double w, double dx, double dy) {
+// at most 1e-10.  Called by a warp; isum, eprev and has are the controller's
+// state, which the caller stores.
+__device__ __forceinline__ double primal_weight(const Scalars *S, double w, double dx, double dy, double &isum, double &eprev,
+                                                int &has) {
     if (!(dx > 1e-10 && dy > 1e-10)) return w;
-    if (S->pw_kp == 0.5 && S->pw_ki == 0.0 && S->pw_kd == 0.0) return exp(0.5 * log(dy / dx) + 0.5 * log(w));
-    const double e = log(w * dx / dy);
-    S->pw_isum += e;
-    const double de = S->pw_has ? e - S->pw_eprev : 0.0;
-    S->pw_eprev = e;
-    S->pw_has = 1;
-    return exp(log(w) - (S->pw_kp * e + S->pw_ki * S->pw_isum + S->pw_kd * de));
+    const bool odd = threadIdx.x & 1;
+    if (S->pw_kp == 0.5 && S->pw_ki == 0.0 && S->pw_kd == 0.0) {
+        const double lg = log(odd ? w : dy / dx);
+        return exp(0.5 * lane_val(lg, 0) + 0.5 * lane_val(lg, 1));
+    }
+    const double lg = log(odd ? w : w * dx / dy);
+    const double e = lane_val(lg, 0);
+    isum += e;
+    const double de = has ? e - eprev : 0.0;
+    eprev = e;
+    has = 1;
+    return exp(lane_val(lg, 1) - (S->pw_kp * e + S->pw_ki * isum + S->pw_kd * de));
 }
 
 // Residual-balance guard: a larger omega is a larger dual step, which works on
@@ -1226,148 +1284,174 @@ __device__ double guard_weight(const Scalars *S, double w, double wn, double rel
     return wn;
 }
 
-__global__ void k_control(Bufs b, int mode, int k_lps) {
-    const int inst = blockIdx.x * blockDim.x + threadIdx.x;
-    if (inst >= k_lps) return;
+// the evaluation's decision for LP `inst`, by a whole warp
+__device__ void control_lp(const Bufs &b, int mode, int inst) {
     Scalars *S = b.S + inst;
-    S->action = ACT_NONE;
-    const bool live = (mode == 0) ? (S->status == NEEDS_INIT) : (S->status == RUNNING);
-    if (!live) return;
+    const int lane = threadIdx.x & 31;
+    const bool first = lane == 0;
+    const int status = S->status;
     const double *T = b.red + (size_t)inst * kPart;
     const double w = S->omega;
+    __syncwarp();
+    if (first) S->action = ACT_NONE;
+    if (mode == 0 ? status != NEEDS_INIT : status != RUNNING) return;
+    // lanes 4 c .. 4 c + 3: the quotients of candidate c
+    const double *Ta = T + (lane >> 2 & 1) * kSlots;
+    double num, den;
+    {
+        const double po = Ta[CX], dob = Ta[QY] + Ta[BND], g = po - dob;
+        const int q = lane & 3;
+        num = q == 0 ? Ta[RPU] : q == 1 ? Ta[RDU] : q == 2 ? fabs(g) : Ta[RD2];
+        den = q == 0 ? 1.0 + S->q_inf : q == 1 ? 1.0 + S->c_inf : q == 2 ? 1.0 + fabs(po) + fabs(dob) : w * w;
+        num = num / den;
+        den = sqrt(w * w * Ta[RP2] + num + g * g);   // the weighted KKT error where q = 3
+    }
     double K[2], rel[2][3], gap[2], pobj[2], dobj[2];
+#pragma unroll
     for (int cnd = 0; cnd < 2; cnd++) {
         const double *a = T + cnd * kSlots;
         pobj[cnd] = a[CX];
         dobj[cnd] = a[QY] + a[BND];
         gap[cnd] = pobj[cnd] - dobj[cnd];
-        K[cnd] = kkt_w(a[RP2], a[RD2], gap[cnd], w);
-        rel[cnd][0] = a[RPU] / (1.0 + S->q_inf);
-        rel[cnd][1] = a[RDU] / (1.0 + S->c_inf);
-        rel[cnd][2] = fabs(gap[cnd]) / (1.0 + fabs(pobj[cnd]) + fabs(dobj[cnd]));
+#pragma unroll
+        for (int q = 0; q < 3; q++) rel[cnd][q] = lane_val(num, 4 * cnd + q);
+        K[cnd] = lane_val(den, 4 * cnd + 3);
     }
+    const int algo = S->algo, metric = S->metric;
+    auto report = [&](int cnd) {
+        S->rel_p = rel[cnd][0]; S->rel_d = rel[cnd][1]; S->rel_g = rel[cnd][2];
+        S->abs_p = T[cnd * kSlots + RPU]; S->pobj = pobj[cnd]; S->dobj = dobj[cnd];
+    };
+    auto stop = [&](int st) { S->status = st; b.status[inst] = st; };
     if (mode == 0) {                     // initial anchor (no residual yet for the fixed-point metric)
-        S->kkt_anchor = (S->algo == ALG_HALPERN && S->metric != METRIC_KKT) ? INFINITY : K[0];
+        if (!first) return;
+        S->kkt_anchor = (algo == ALG_HALPERN && metric != METRIC_KKT) ? INFINITY : K[0];
         S->kkt_prev = INFINITY;
-        S->rel_p = rel[0][0]; S->rel_d = rel[0][1]; S->rel_g = rel[0][2];
-        S->abs_p = T[RPU]; S->pobj = pobj[0]; S->dobj = dobj[0];
-        S->status = isfinite(K[0]) ? RUNNING : NUMERIC;
-        b.status[inst] = S->status;
+        report(0);
+        stop(isfinite(K[0]) ? RUNNING : NUMERIC);
         return;
     }
-    const int n_eval = S->n_eval;
-    if (S->k_base + n_eval > S->max_iter) {   // partial block: limit reached inside it
-        S->status = ITER_LIMIT;
-        b.status[inst] = S->status;
+    const int n_eval = S->n_eval, max_iter = S->max_iter, k = S->k_base + n_eval, j = S->j_base + n_eval;
+    if (k > max_iter) {                  // partial block: limit reached inside it
+        if (first) stop(ITER_LIMIT);
         return;
     }
-    const int k = S->k_base + n_eval;
-    const int j = S->j_base + n_eval;
-    S->evals += 1;
-    S->inv_j = S->adaptive ? (S->wsum > 0.0 ? S->inv_wsum : 0.0) : S->inv_next;
-    S->k_base = k;
-    if (S->algo == ALG_HALPERN) {
+    const int evals = S->evals + 1;
+    const double anchor = S->kkt_anchor, prev = S->kkt_prev, eta = S->eta, tol = S->tol, stop_abs = S->stop_abs;
+    const double ad_eta = S->ad_eta;
+    double isum = S->pw_isum, eprev = S->pw_eprev;
+    int has = S->pw_has;
+    __syncwarp();
+    if (first) {
+        S->evals = evals;
+        S->inv_j = S->adaptive ? (S->wsum > 0.0 ? S->inv_wsum : 0.0) : S->inv_next;
+        S->k_base = k;
+    }
+    if (algo == ALG_HALPERN) {
         // candidate 0 = last map output; fixed-point residual terms in the second record
         const double fx2 = T[kSlots + DX2], fy2 = T[kSlots + DY2];
         if (!isfinite(K[0]) || !isfinite(fx2) || !isfinite(fy2)) {
-            S->status = NUMERIC;
-            b.status[inst] = S->status;
+            if (first) stop(NUMERIC);
             return;
         }
-        S->rel_p = rel[0][0]; S->rel_d = rel[0][1]; S->rel_g = rel[0][2];
-        S->abs_p = T[RPU]; S->pobj = pobj[0]; S->dobj = dobj[0];
-        if (S->stop_abs > 0.0 ? (T[RPU] <= S->stop_abs) : (fmax(rel[0][0], fmax(rel[0][1], rel[0][2])) <= S->tol)) {
-            S->status = OPTIMAL;
-            S->which = 0;
-            b.status[inst] = S->status;
+        if (first) report(0);
+        if (stop_abs > 0.0 ? (T[RPU] <= stop_abs) : (fmax(rel[0][0], fmax(rel[0][1], rel[0][2])) <= tol)) {
+            if (first) { stop(OPTIMAL); S->which = 0; }
             return;
         }
-        if (S->evals % kInfeasEvery == 0) {
+        if (evals % kInfeasEvery == 0) {
             const double obj = T[kSlots + QY] + T[kSlots + BND];
             const double viol = fmax(T[kSlots + RPU], T[kSlots + RDU]);
             if (obj > 0.0 && viol <= kInfeasEps * obj) {
-                S->status = INFEASIBLE;
-                b.status[inst] = S->status;
+                if (first) stop(INFEASIBLE);
                 return;
             }
         }
-        const double cross = (S->metric == METRIC_FPRP) ? T[kSlots + CX] : 0.0;
-        const double r = (S->metric == METRIC_KKT) ? K[0] : sqrt(fmax(w * fx2 + fy2 / w - 2.0 * S->eta * cross, 0.0));
-        const bool restart = (r <= 0.2 * S->kkt_anchor) ||
-                             (r <= 0.8 * S->kkt_anchor && r > S->kkt_prev) ||
-                             ((double)j >= 0.36 * (double)k);
+        const double cross = (metric == METRIC_FPRP) ? T[kSlots + CX] : 0.0;
+        const double r = (metric == METRIC_KKT) ? K[0] : sqrt(fmax(w * fx2 + fy2 / w - 2.0 * eta * cross, 0.0));
+        const bool restart = (r <= 0.2 * anchor) || (r <= 0.8 * anchor && r > prev) || ((double)j >= 0.36 * (double)k);
         if (restart) {
-            const double dx = sqrt(T[DX2]), dy = sqrt(T[DY2]);
-            const double wn = guard_weight(S, w, primal_weight(S, w, dx, dy), rel[0][0], rel[0][1]);
-            S->omega = wn;
-            S->kkt_anchor = (S->metric == METRIC_KKT) ? kkt_w(T[RP2], T[RD2], gap[0], wn)
-                                                      : sqrt(fmax(wn * fx2 + fy2 / wn - 2.0 * S->eta * cross, 0.0));
-            S->kkt_prev = INFINITY;
-            S->j_base = 0;
-            S->restarts += 1;
-            S->tau = S->eta / wn;
-            S->sigma = S->eta * wn;
-            S->action = ACT_RESTART;
-        } else {
+            const double root = sqrt(T[(lane & 1) ? DY2 : DX2]);
+            const double dx = lane_val(root, 0), dy = lane_val(root, 1);
+            const double wn = guard_weight(S, w, primal_weight(S, w, dx, dy, isum, eprev, has), rel[0][0], rel[0][1]);
+            // tau and the anchor's quotient side by side
+            const double quo = ((lane & 1) ? (metric == METRIC_KKT ? T[RD2] : fy2) : eta) /
+                               ((lane & 1) && metric == METRIC_KKT ? wn * wn : wn);
+            const double tau = lane_val(quo, 0), part = lane_val(quo, 1);
+            const double an = metric == METRIC_KKT ? sqrt(wn * wn * T[RP2] + part + gap[0] * gap[0])
+                                                   : sqrt(fmax(wn * fx2 + part - 2.0 * eta * cross, 0.0));
+            if (first) {
+                S->omega = wn;
+                S->pw_isum = isum; S->pw_eprev = eprev; S->pw_has = has;
+                S->kkt_anchor = an;
+                S->kkt_prev = INFINITY;
+                S->j_base = 0;
+                S->restarts += 1;
+                S->tau = tau;
+                S->sigma = eta * wn;
+                S->action = ACT_RESTART;
+            }
+        } else if (first) {
             S->kkt_prev = r;
             S->j_base = j;
         }
-        if (k >= S->max_iter) {
-            S->status = ITER_LIMIT;
-            b.status[inst] = S->status;
-        }
+        if (first && k >= max_iter) stop(ITER_LIMIT);
         return;
     }
     if (!isfinite(K[0]) || !isfinite(K[1])) {
-        S->status = NUMERIC;
-        b.status[inst] = S->status;
+        if (first) stop(NUMERIC);
         return;
     }
+#pragma unroll
     for (int cnd = 0; cnd < 2; cnd++) {
         const double mx = fmax(rel[cnd][0], fmax(rel[cnd][1], rel[cnd][2]));
-        if (mx <= S->tol) {
-            S->status = OPTIMAL;
-            S->which = cnd;
-            S->action = ACT_FINISH;
-            S->rel_p = rel[cnd][0]; S->rel_d = rel[cnd][1]; S->rel_g = rel[cnd][2];
-            S->abs_p = T[cnd * kSlots + RPU]; S->pobj = pobj[cnd]; S->dobj = dobj[cnd];
-            b.status[inst] = S->status;
+        if (mx <= tol) {
+            if (first) { S->which = cnd; S->action = ACT_FINISH; report(cnd); stop(OPTIMAL); }
             return;
         }
     }
-    S->rel_p = rel[0][0]; S->rel_d = rel[0][1]; S->rel_g = rel[0][2];
-    S->abs_p = T[RPU]; S->pobj = pobj[0]; S->dobj = dobj[0];
+    if (first) report(0);
     const int cand = (K[1] < K[0]) ? 1 : 0;
-    const double kc = K[cand];
-    const bool restart = (kc <= 0.2 * S->kkt_anchor) ||
-                         (kc <= 0.8 * S->kkt_anchor && kc > S->kkt_prev) ||
-                         ((double)j >= 0.36 * (double)k);
+    const double kc = cand ? K[1] : K[0];
+    const bool restart = (kc <= 0.2 * anchor) || (kc <= 0.8 * anchor && kc > prev) || ((double)j >= 0.36 * (double)k);
     if (restart) {
         const double *a = T + cand * kSlots;
-        const double dx = sqrt(a[DX2]), dy = sqrt(a[DY2]);
-        const double wn = primal_weight(S, w, dx, dy);
-        S->omega = wn;
-        S->kkt_anchor = kkt_w(a[RP2], a[RD2], gap[cand], wn);
-        S->kkt_prev = INFINITY;
-        S->j_base = 0;
-        S->restarts += 1;
-        S->tau = S->eta / wn;
-        S->sigma = S->eta * wn;
-        S->cand = cand;
-        S->wsum = 0.0;
-        S->inv_wsum = 0.0;
-        S->ad_tau = S->ad_eta / wn;
-        S->ad_sigma = S->ad_eta * wn;
-        S->action = ACT_RESTART;
-    } else {
+        const double root = sqrt(a[(lane & 1) ? DY2 : DX2]);
+        const double dx = lane_val(root, 0), dy = lane_val(root, 1);
+        const double wn = primal_weight(S, w, dx, dy, isum, eprev, has);
+        const double quo = ((lane & 3) == 0 ? eta : (lane & 3) == 1 ? a[RD2] : ad_eta) / ((lane & 3) == 1 ? wn * wn : wn);
+        const double tau = lane_val(quo, 0), part = lane_val(quo, 1), ad_tau = lane_val(quo, 2);
+        const double g = cand ? gap[1] : gap[0];
+        const double an = sqrt(wn * wn * a[RP2] + part + g * g);
+        if (first) {
+            S->omega = wn;
+            S->pw_isum = isum; S->pw_eprev = eprev; S->pw_has = has;
+            S->kkt_anchor = an;
+            S->kkt_prev = INFINITY;
+            S->j_base = 0;
+            S->restarts += 1;
+            S->tau = tau;
+            S->sigma = eta * wn;
+            S->cand = cand;
+            S->wsum = 0.0;
+            S->inv_wsum = 0.0;
+            S->ad_tau = ad_tau;
+            S->ad_sigma = ad_eta * wn;
+            S->action = ACT_RESTART;
+        }
+    } else if (first) {
         S->kkt_prev = kc;
         S->j_base = j;
     }
-    S->inv_next = 1.0 / (double)(S->j_base + n_eval);
-    if (k >= S->max_iter) {
-        S->status = ITER_LIMIT;
-        b.status[inst] = S->status;
-    }
+    if (!first) return;
+    S->inv_next = 1.0 / (double)((restart ? 0 : j) + n_eval);
+    if (k >= max_iter) stop(ITER_LIMIT);
+}
+
+constexpr int kControlThreads = 128;   // four LPs per CTA
+__global__ void __launch_bounds__(kControlThreads) k_control(Bufs b, int mode, int k_lps) {
+    const int inst = (int)(blockIdx.x * kControlThreads + threadIdx.x) >> 5;
+    if (inst < k_lps) control_lp(b, mode, inst);
 }
 
 // Average variant: restart (current <- candidate, anchor <- candidate,
@@ -1608,6 +1692,8 @@ struct Layout {
     size_t chunks_p, chunks_d, ctas_p, ctas_d;
     // period-strided groups: k per group and slot records (row kernels)
     size_t A_sk, AT_sk, A_sl, AT_sl;
+    // resident block kernel: tiles, their split over warps, tagged vectors, iteration count, timing stamps
+    size_t tiles, warps, xt, yt, blk_seq, stamp;
     // lanes sessions: contiguous staging for one LP's vectors (4 (n + m) doubles:
     // the seven vectors a result may download)
     size_t lane_stage;
@@ -1663,6 +1749,12 @@ struct uc_session {
     // period-strided 16-row groups read from slot records (row kernels, K = 1)
     bool strided = false;
     int64_t strided_rows_A = 0, strided_rows_AT = 0;
+    // resident block kernel: possible for this session; used by the current tables
+    bool block_able = false, block = false;
+    int sms = 0, blk_smem_max = 0;          // SMs, shared memory per CTA
+    int blk_ctas = 0, blk_threads = 0, blk_smem = 0;
+    uc::dev::BlockPlan plan{};
+    unsigned long long *h_stamp = nullptr;   // pinned [2][2]: timed iteration's bounds of each graph
     // staged iteration kernels
     bool staged = false;
     int stages = 4;
@@ -1688,6 +1780,7 @@ struct uc_session {
         for (auto e : ev) if (e) cudaEventDestroy(e);
         for (auto &row : tev) for (auto e : row) if (e) cudaEventDestroy(e);
         if (h_status) cudaFreeHost(h_status);
+        if (h_stamp) cudaFreeHost(h_stamp);
         if (D) {
             if (o.free) o.free(D, bytes, (void *)s, o.alloc_ctx);
             else cudaFreeAsync(D, s);
@@ -2069,7 +2162,7 @@ static void launch_eval(uc_session &X, cudaStream_t s, int mode) {
         else k_eval<double, 4><<<grid, kThreads, 0, s>>>(X.dse, X.b, mode);
     }
     k_reduce<<<X.k * kPart, kThreads, 0, s>>>(X.drg, X.b, mode);
-    k_control<<<(X.k + 127) / 128, 128, 0, s>>>(X.b, mode, X.k);
+    k_control<<<(32 * X.k + kControlThreads - 1) / kControlThreads, kControlThreads, 0, s>>>(X.b, mode, X.k);
 }
 
 // iteration kernels of the session's algorithm
@@ -2207,6 +2300,36 @@ static void launch_adaptive_norm(uc_session &X, cudaStream_t s) {
     k_ad_src0<<<1, 1, 0, s>>>(X.b);
 }
 
+using BlockKernel = void (*)(BlockPlan, Bufs);
+template <typename VT>
+static BlockKernel block_kernel_vt(int threads, bool one) {
+    if (threads <= 256) return one ? k_block<VT, 256, true> : k_block<VT, 256, false>;
+    return one ? k_block<VT, 1024, true> : k_block<VT, 1024, false>;
+}
+static BlockKernel block_kernel(const uc_session &X, int threads) {
+    return X.vb == 32 ? block_kernel_vt<float>(threads, X.k == 1) : block_kernel_vt<double>(threads, X.k == 1);
+}
+static int block_head(const uc_session &X) {
+    return (int)(sizeof(BlockLp) * X.k + sizeof(double2) * (X.k == 1 ? X.o.n_eval + 1 : 0));
+}
+
+// all n_eval iterations of a block (cooperative: the CTAs wait on one another,
+// so all of them are resident)
+static void launch_block(uc_session &X, cudaStream_t s) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(X.blk_ctas);
+    cfg.blockDim = dim3(X.blk_threads);
+    cfg.dynamicSmemBytes = X.blk_smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, block_kernel(X, X.blk_threads), X.plan, X.b);
+    if (e != cudaSuccess && X.launch_err == cudaSuccess) X.launch_err = e;
+}
+
 static int capture(uc_session &X, int gi) {
     cudaStream_t s = X.s;
     const bool timing = X.o.kernel_timing != 0;
@@ -2219,7 +2342,10 @@ static int capture(uc_session &X, int gi) {
     // the timed pair is a mid-block iteration: steady-state L2 contents, and
     // only the event nodes around it break the programmatic overlap
     const int timed_it = X.o.n_eval / 2;
-    for (int it = 0; it < X.o.n_eval; it++) {
+    if (X.block) launch_block(X, s);
+    if (X.block && timing && err == cudaSuccess)
+        err = cudaMemcpyAsync(X.h_stamp + 2 * gi, X.plan.stamp, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s);
+    for (int it = 0; !X.block && it < X.o.n_eval; it++) {
         if (X.adaptive) {
             launch_adaptive(X, s, it, [&](int e) { if (it == timed_it) rec(e); });
             continue;
@@ -2255,7 +2381,8 @@ static int capture(uc_session &X, int gi) {
 static int launch_direct(uc_session &X) {
     cudaStream_t s = X.s;
     const Bufs &b = X.b;
-    for (int it = 0; it < X.o.n_eval; it++) {
+    if (X.block) launch_block(X, s);
+    for (int it = 0; !X.block && it < X.o.n_eval; it++) {
         if (X.adaptive) {
             launch_adaptive(X, s, it, [](int) {});
             continue;
@@ -2316,8 +2443,9 @@ static void build_tables(const uc_session &X, const std::vector<char> &mask, std
         const int eq_end = X.m_eq[0];
         for (int64_t s = 0; s < X.Nr; s += rows) sp.push_back({0, (int)s, (int)std::min<int64_t>(s + rows, X.Nr), 0, 1});
         for (int64_t s = 0; s < X.Mr; s += rows) sd.push_back({0, (int)s, (int)std::min<int64_t>(s + rows, X.Mr), eq_end, 1});
-        for (int64_t s = 0; s < X.Mr; s += kEvalRows) se.push_back({0, (int)s, (int)std::min<int64_t>(s + kEvalRows, X.Mr), eq_end << 1, 1});
-        for (int64_t s = 0; s < X.Nr; s += kEvalRows) se.push_back({0, (int)s, (int)std::min<int64_t>(s + kEvalRows, X.Nr), 1, 1});
+        const int er = eval_rows(X.Mr + X.Nr);
+        for (int64_t s = 0; s < X.Mr; s += er) se.push_back({0, (int)s, (int)std::min<int64_t>(s + er, X.Mr), eq_end << 1, 1});
+        for (int64_t s = 0; s < X.Nr; s += er) se.push_back({0, (int)s, (int)std::min<int64_t>(s + er, X.Nr), 1, 1});
         if (se.empty()) se.push_back({0, 0, 0, 0, 1});
         for (int i = 0; i < X.k; i++) ranges[i] = {i * (int)se.size(), (i + 1) * (int)se.size()};
         for (int64_t s = 0; s < X.Nr; s += X.cta) sa.push_back({0, (int)s, (int)std::min<int64_t>(s + X.cta, X.Nr), 0, 1});
@@ -2338,8 +2466,9 @@ static void build_tables(const uc_session &X, const std::vector<char> &mask, std
         const int eq_end = (int)(r0 + X.m_eq[i]);
         for (int64_t s = r0; s < r1; s += cta) sd.push_back({i, (int)s, (int)std::min<int64_t>(s + cta, r1), eq_end, rpt});
         ranges[i].eval_begin = (int)se.size();
-        for (int64_t s = r0; s < r1; s += kEvalRows) se.push_back({i, (int)s, (int)std::min<int64_t>(s + kEvalRows, r1), eq_end << 1, 1});
-        for (int64_t s = c0; s < cl; s += kEvalRows) se.push_back({i, (int)s, (int)std::min<int64_t>(s + kEvalRows, cl), 1, 1});
+        const int er = eval_rows(c1 - c0 + r1 - r0);
+        for (int64_t s = r0; s < r1; s += er) se.push_back({i, (int)s, (int)std::min<int64_t>(s + er, r1), eq_end << 1, 1});
+        for (int64_t s = c0; s < cl; s += er) se.push_back({i, (int)s, (int)std::min<int64_t>(s + er, cl), 1, 1});
         for (int64_t s = cl; s < c1; s += kThreads / 32) se.push_back({i, (int)s, (int)std::min<int64_t>(s + kThreads / 32, c1), 1, 0});
         if (se.size() == (size_t)ranges[i].eval_begin) se.push_back({i, 0, 0, 0, 1});
         ranges[i].eval_end = (int)se.size();
@@ -2348,6 +2477,78 @@ static void build_tables(const uc_session &X, const std::vector<char> &mask, std
     n_sac = (int)sac.size();
     sa = sac;
     sa.insert(sa.end(), sd.begin(), sd.end());
+}
+
+// Tiles of the resident block kernel for the LPs in `mask`, dealt to the warps of
+// at most one CTA per SM: primal tiles, longest rows first, to the warps in turn
+// over the CTAs, dual tiles in turn from the last warp back, so that a warp has
+// tiles of one phase while there are warps enough and the longest rows get a warp
+// of their own.  Sets X.block: the tiles fit into the CTAs' shared memory.
+static void plan_block(uc_session &X, const std::vector<char> &mask, std::vector<BlockTile> &tiles,
+                       std::vector<BlockWarp> &warps) {
+    tiles.clear();
+    warps.clear();
+    X.block = false;
+    if (!X.block_able) return;
+    std::vector<BlockTile> t[2];   // dual, primal
+    int64_t bytes = 0;
+    for (int i = 0; i < X.k; i++) {
+        if (!mask[i]) continue;
+        const PsData &v = *X.Pd[i];
+        const int n = v.n(), m = v.m(), nl = v.long_cols, m_eq = X.m_eq[i];
+        auto cut = [&](const Csr &M, int a, int b, int64_t base, int aux, bool primal) {
+            for (int s = a; s < b; s += kTileRows) {
+                const int e = std::min(b, s + kTileRows);
+                int kmax = 0;
+                for (int r = s; r < e; r++) kmax = std::max(kmax, M.rowptr[r + 1] - M.rowptr[r]);
+                t[primal].push_back(BlockTile{(int)(base + s), e - s, i, aux, kmax, 0, 0, 0});
+                bytes += tile_bytes(kmax, primal);
+            }
+        };
+        cut(v.AT, 0, n - nl, X.coff[i], 0, true);
+        for (int j = n - nl; j < n; j++) {
+            const int kmax = (v.AT.rowptr[j + 1] - v.AT.rowptr[j] + 31) / 32;
+            t[1].push_back(BlockTile{(int)(X.coff[i] + j), 1, i, 0, kmax, 0, 1, 0});
+            bytes += tile_bytes(kmax, true);
+        }
+        cut(v.A, 0, m, X.roff[i], (int)X.roff[i] + m_eq, false);
+        if (bytes > (int64_t)X.sms * X.blk_smem_max) return;
+    }
+    const int64_t np = t[1].size(), nd = t[0].size();
+    if (np == 0 || nd == 0) return;
+    const int nc = (int)std::min<int64_t>(X.sms, std::max(np, nd));
+    const int W = (int)std::min<int64_t>(32, (np + nd + nc - 1) / nc);
+    const int64_t S = (int64_t)nc * W;
+    std::vector<std::vector<const BlockTile *>> mine[2];
+    for (int ph = 0; ph < 2; ph++) {
+        mine[ph].resize(S);
+        std::stable_sort(t[ph].begin(), t[ph].end(), [](const BlockTile &a, const BlockTile &b) { return a.kmax > b.kmax; });
+        for (int64_t i = 0; i < (int64_t)t[ph].size(); i++) mine[ph][ph ? i % S : S - 1 - i % S].push_back(&t[ph][i]);
+    }
+    const int head = block_head(X);
+    int most = 0;
+    for (int c = 0; c < nc; c++) {
+        int64_t at = 0;
+        for (int w = 0; w < W; w++) {
+            const int64_t slot = (int64_t)w * nc + c;
+            warps.push_back(BlockWarp{(int)tiles.size(), (int)mine[1][slot].size(), (int)mine[0][slot].size(), 0});
+            for (int ph = 1; ph >= 0; ph--)
+                for (const BlockTile *p : mine[ph][slot]) {
+                    tiles.push_back(*p);
+                    tiles.back().smem = (int)at;
+                    at += tile_bytes(p->kmax, ph == 1);
+                    if (head + at > X.blk_smem_max) return;
+                }
+        }
+        most = std::max(most, (int)at);
+    }
+    X.plan.head = head;
+    X.plan.nlps = X.k;
+    X.plan.n_eval = X.o.n_eval;
+    X.blk_ctas = nc;
+    X.blk_threads = 32 * W;
+    X.blk_smem = head + most;
+    X.block = true;
 }
 
 // Chunk lists of the staged kernels for the LPs in `mask`: rows are cut into
@@ -2415,6 +2616,11 @@ static int retable(uc_session &X, const std::vector<char> &mask) {
     if (!rc) rc = up(L.segs_e, se.data(), sizeof(Seg) * se.size());
     if (!rc) rc = up(L.segs_a, sa.data(), sizeof(Seg) * sa.size());
     if (!rc) rc = up(L.ranges, ranges.data(), sizeof(InstRange) * ranges.size());
+    std::vector<BlockTile> tiles;
+    std::vector<BlockWarp> warps;
+    plan_block(X, mask, tiles, warps);
+    if (!rc && X.block) rc = up(L.tiles, tiles.data(), sizeof(BlockTile) * tiles.size());
+    if (!rc && X.block) rc = up(L.warps, warps.data(), sizeof(BlockWarp) * warps.size());
     std::vector<Chunk> cp, cd;
     std::vector<int> gp, gd;
     if (X.staged) {
@@ -2586,6 +2792,24 @@ static int session_create(const PsData *const *Pp, const std::shared_ptr<const P
     X->n_sp = X->cap_sp = (int)sp.size(); X->n_sd = X->cap_sd = (int)sd.size();
     X->n_se = X->cap_se = (int)se.size(); X->n_sa = X->cap_sa = (int)sa.size();
 
+    // resident block kernel: Halpern row sessions
+    std::vector<BlockTile> tiles;
+    std::vector<BlockWarp> warps;
+    {
+        int dev = 0, coop = 0;
+        UC_CUDA(cudaGetDevice(&dev));
+        UC_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
+        UC_CUDA(cudaDeviceGetAttribute(&X->sms, cudaDevAttrMultiProcessorCount, dev));
+        UC_CUDA(cudaDeviceGetAttribute(&X->blk_smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+        X->blk_smem_max -= 1024;   // the kernel's static part
+        X->block_able = coop && o.spmv_kernel == 0 && X->algo == ALG_HALPERN && X->K == 1 && k <= kBlockMaxLps &&
+                        o.n_eval <= kBlockMaxEval;
+        if (X->block_able)
+            for (int nt : {256, 1024})
+                UC_CUDA(cudaFuncSetAttribute(block_kernel(*X, nt), cudaFuncAttributeMaxDynamicSharedMemorySize, X->blk_smem_max));
+        plan_block(*X, all, tiles, warps);
+        if (k == 1 && !X->block) X->block_able = false;   // no subset of its LPs fits either
+    }
     Layout &L = X->L;
     size_t off = 0;
     // 16 bytes of slack after every array: the staged kernels' copies round
@@ -2615,10 +2839,23 @@ static int session_create(const PsData *const *Pp, const std::shared_ptr<const P
     L.inv_Dc = take(N * 8); L.lkey = take(N * 8); L.ukey = take(N * 8);
     L.q = take(M * 8); L.Dr = take(M * 8); L.inv_Dr = take(M * 8);
     L.x_init = take(N * 8); L.y_init = take(M * 8); L.S_init = take(sizeof(Scalars) * k);
+    {   // tables for any subset of the LPs: a tile per 32 rows or columns begun, or per long column
+        int64_t nt = 0;
+        for (int i = 0; i < k && X->block_able; i++) {
+            const PsData &p = *X->Pd[i];
+            nt += (p.n() + kTileRows - 1) / kTileRows + (p.m() + kTileRows - 1) / kTileRows + p.long_cols;
+        }
+        L.tiles = take(sizeof(BlockTile) * nt);
+        L.warps = take(X->block_able ? sizeof(BlockWarp) * 32 * X->sms : 0);
+    }
     L.upload_end = off;
     L.x0 = take(N * 8); L.x1 = take(N * 8); L.y0 = take(M * 8); L.y1 = take(M * 8);
     L.xsum = take(N * 8); L.ysum = take(M * 8); L.xa = take(N * 8); L.ya = take(M * 8);
     L.xret = take(N * 8); L.yret = take(M * 8);
+    L.xt = take(X->block_able ? N * 16 : 0);
+    L.yt = take(X->block_able ? M * 16 : 0);
+    L.blk_seq = take(sizeof(unsigned));
+    L.stamp = take(2 * sizeof(unsigned long long));
     L.part = take(sizeof(double) * kPart * X->n_se * X->K);
     L.adp = take(X->adaptive ? sizeof(double) * (size_t)((Nr + kAdThreads - 1) / kAdThreads + 2 * ((Mr + kAdThreads - 1) / kAdThreads)) : 0);
     L.lane_stage = take(X->K > 1 ? (size_t)4 * (Nr + Mr) * 8 : 0);
@@ -2674,6 +2911,10 @@ static int session_create(const PsData *const *Pp, const std::shared_ptr<const P
         put(st, L.segs_e, se.data(), X->n_se);
         put(st, L.segs_a, sa.data(), X->n_sa);
         put(st, L.ranges, ranges.data(), k);
+        if (X->block) {
+            put(st, L.tiles, tiles.data(), tiles.size());
+            put(st, L.warps, warps.data(), warps.size());
+        }
         put(st, L.chunks_p, cp.data(), cp.size()); put(st, L.chunks_d, cd.data(), cd.size());
         put(st, L.ctas_p, gp.data(), gp.size()); put(st, L.ctas_d, gd.data(), gd.size());
         // Halpern weights, computed as the oracle's Halpern step computes them: w = (j+1)/(j+2), 1 - w
@@ -2732,6 +2973,15 @@ static int session_create(const PsData *const *Pp, const std::shared_ptr<const P
     b.xa = (double *)(D + L.xa); b.ya = (double *)(D + L.ya);
     b.xret = (double *)(D + L.xret); b.yret = (double *)(D + L.yret);
     b.part = (double *)(D + L.part);
+    b.blk_seq = (unsigned *)(D + L.blk_seq);
+    b.n_eval = o.n_eval;
+    X->plan.tiles = (const BlockTile *)(D + L.tiles);
+    X->plan.warps = (const BlockWarp *)(D + L.warps);
+    X->plan.seq = b.blk_seq;
+    X->plan.xt = (ulonglong2 *)(D + L.xt);
+    X->plan.yt = (ulonglong2 *)(D + L.yt);
+    X->plan.stamp = o.kernel_timing ? (unsigned long long *)(D + L.stamp) : nullptr;
+    X->plan.stamp_it = o.n_eval / 2;
     b.S = (Scalars *)(D + L.S);
     b.status = (int *)(D + L.status);
     X->dsp = (const Seg *)(D + L.segs_p); X->dsd = (const Seg *)(D + L.segs_d);
@@ -2742,11 +2992,21 @@ static int session_create(const PsData *const *Pp, const std::shared_ptr<const P
     // nothing runs until the first reset: mark every LP finished-as-idle
     UC_CUDA(cudaMemsetAsync(D + L.S, 0xff, sizeof(Scalars) * k, s));   // status -1: idle
     UC_CUDA(cudaMemsetAsync(D + L.status, 0xff, sizeof(int) * k, s));
+    UC_CUDA(cudaMemsetAsync(D + L.blk_seq, 0, sizeof(unsigned), s));
+    if (X->block_able) {   // tag 0: no iteration's
+        UC_CUDA(cudaMemsetAsync(D + L.xt, 0, N * 16, s));
+        UC_CUDA(cudaMemsetAsync(D + L.yt, 0, M * 16, s));
+    }
+    UC_CUDA(cudaMemsetAsync(D + L.stamp, 0, 2 * sizeof(unsigned long long), s));
     UC_CUDA(cudaHostAlloc((void **)&X->h_status, sizeof(int) * k, cudaHostAllocDefault));
     for (int i = 0; i < k; i++) X->h_status[i] = -1;
     X->active.assign(k, 0);
     const bool timing = o.kernel_timing != 0;
     for (auto &e : X->ev) UC_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    if (X->block_able && timing) {
+        UC_CUDA(cudaHostAlloc((void **)&X->h_stamp, 4 * sizeof(unsigned long long), cudaHostAllocDefault));
+        std::memset(X->h_stamp, 0, 4 * sizeof(unsigned long long));
+    }
     if (o.use_graph) {
         for (int gi = 0; gi < 2; gi++) {
             if (timing)
@@ -2857,7 +3117,7 @@ static int session_run(uc_session &X, int max_replays) {
             UC_CUDA(cudaEventRecord(X.ev[launched & 3], s));
             launched++;
             X.polls++;
-            X.launches += X.adaptive ? 3LL * X.o.n_eval + 6 : 2LL * X.o.n_eval + 4;
+            X.launches += X.block ? 5 : X.adaptive ? 3LL * X.o.n_eval + 6 : 2LL * X.o.n_eval + 4;
         }
         if (checked >= launched) break;
         UC_CUDA(cudaEventSynchronize(X.ev[checked & 3]));
@@ -2883,7 +3143,14 @@ static int session_run(uc_session &X, int max_replays) {
                 }
             }
         }
-        if (timing && !done) {
+        if (timing && !done && X.block) {
+            // the halves of an iteration overlap: its time is split by their FP64 instructions
+            const volatile unsigned long long *t = X.h_stamp + 2 * gi;
+            if (t[0] && t[1] > t[0]) {
+                const double ms = (double)(t[1] - t[0]) * 1e-6, p = (double)(X.Z + 4 * X.N), d = (double)(X.Z + 4 * X.M);
+                X.tp_sum += ms * p / (p + d); X.td_sum += ms * d / (p + d); X.timed++;
+            }
+        } else if (timing && !done) {
             float a = 0.f, c = 0.f;
             if (cudaEventElapsedTime(&a, X.tev[gi][0], X.tev[gi][1]) == cudaSuccess &&
                 cudaEventElapsedTime(&c, X.tev[gi][1], X.tev[gi][2]) == cudaSuccess) {
@@ -2984,7 +3251,8 @@ static int session_result(uc_session &X, int i, uc_result **out) {
     else if (S.status == INFEASIBLE) status = UC_EINFEASIBLE;
     else if (S.status == STALLED) {
         status = UC_ECUDA;
-        set_error("a staged iteration kernel stopped waiting for its shared-memory copies");
+        set_error(X.staged ? "a staged iteration kernel stopped waiting for its shared-memory copies"
+                           : "the resident block kernel stopped waiting for another CTA's element");
     }
     else status = X.host_status ? X.host_status : UC_EITERLIMIT;
     o.status = status;

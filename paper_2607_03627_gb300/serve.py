@@ -242,13 +242,14 @@ def sequential_baseline(requests: list[Request], base_problem, tol: float = 1e-4
 def session_bytes_estimate(ps, value_bits: int = 64, max_iter: int = 100_000) -> int:
     """Device bytes of a one-LP session of `ps`, estimated from its sizes: the
     matrix and its transpose (int32 indices, FP64 or FP32 values, row pointers),
-    the period-strided slot records, eight constant and start vectors and ten
-    state vectors per column or row, and the Halpern weight tables."""
+    the period-strided slot records, eight constant and start vectors, ten state
+    vectors and a tagged copy of the iterate per column or row, the resident
+    kernel's tiles, and the Halpern weight tables."""
     n, m, _, nnz = B.uc_presolved_dims(ps)
     vs = 4 if value_bits == 32 else 8
     slot = 8 if value_bits == 32 else 16
-    per_col = 4 + 8 * 8 + 5 * 8 + slot
-    per_row = 4 + 4 * 8 + 5 * 8 + slot
+    per_col = 4 + 8 * 8 + 5 * 8 + slot + 17
+    per_row = 4 + 4 * 8 + 5 * 8 + slot + 17
     tables = 2 * 8 * min(max_iter + 1, 1 << 22)
     return int(1.05 * (2 * nnz * (4 + vs) + n * per_col + m * per_row + tables) + (1 << 20))
 
