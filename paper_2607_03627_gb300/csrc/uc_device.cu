@@ -294,6 +294,29 @@ __device__ __forceinline__ int row_head(const int *__restrict__ ci_arr, const VT
 // The loads of a row are issued before the LP's state is read (the addresses
 // are valid either way), so that read overlaps them instead of heading the
 // chain of dependent loads.  SD: strided groups read their slots (see above).
+// Halpern: an iteration stores x-bar only; its x is the Halpern step from the
+// x-bar of the iteration before (it > 0, v) and the anchor x0: 8 bytes per column
+// less to store (6,049 buses 33.7 -> 33.1 us per iteration, 2,000 buses with the
+// angles eliminated 21.0 -> 19.0; taken before the gathers instead of after them
+// it spills and gives 33.5 and 19.5).  The block's last iteration also writes what
+// the evaluation and the next block read: x, the next x and the map output.
+__device__ __forceinline__ double halpern_x(const Bufs &b, const Scalars *S, int it, int j, double v, double x0) {
+    if (it == 0) return v;
+    double w, w1;
+    halpern_weights(b, S, it - 1, w, w1);
+    return fma(w, v, w1 * x0);
+}
+__device__ __forceinline__ void halpern_store(const Bufs &b, const Scalars *S, int it, int src, int j, double x, double xv, bool keep) {
+    const double xb = fma(2.0, xv, -x);
+    b.xsum[j] = xb;
+    if (!keep) return;
+    double w, w1;
+    halpern_weights(b, S, it, w, w1);
+    b.x[src][j] = x;
+    b.x[src ^ 1][j] = fma(w, xb, w1 * b.xa[j]);
+    b.xret[j] = xv;
+}
+
 // A long column (more than kLongRow entries) gets a warp: the lanes stride over
 // its entries, their partial sums are added in a fixed butterfly order, and
 // lane 0 adds -c and applies the column's update as the one-thread path does.
@@ -316,21 +339,16 @@ __device__ __forceinline__ void primal_long(const Seg &sg, const Bufs &b, int it
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
     if (lane != 0) return;
-    const double xin = ld_stream(b.x[src] + j);
     const long long lk = ld_stream(b.lkey + j), uk = ld_stream(b.ukey + j);
     const double aux = (ALGO == ALG_AVERAGE) ? b.xsum[j] : ld_stream(b.xa + j);
+    const double xin = (ALGO == ALG_AVERAGE) ? ld_stream(b.x[src] + j) : halpern_x(b, S, it, j, it > 0 ? b.xsum[j] : b.x[0][j], aux);
     const double acc = neg_bits(ld_stream(b.c + j)) + part;
     const double xv = clip_keys(fma(S->tau, acc, xin), lk, uk);
     if (ALGO == ALG_AVERAGE) {
         b.x[src ^ 1][j] = xv;
         b.xsum[j] = aux + xv;
     } else {
-        double w, w1;
-        halpern_weights(b, S, it, w, w1);
-        const double xb = fma(2.0, xv, -xin);
-        b.xsum[j] = xb;
-        b.x[src ^ 1][j] = fma(w, xb, w1 * aux);
-        if (keep) b.xret[j] = xv;
+        halpern_store(b, S, it, src, j, xin, xv, keep);
     }
 }
 
@@ -359,7 +377,7 @@ __global__ void __launch_bounds__(BS, 1536 / BS) k_primal(const Seg *__restrict_
 #pragma unroll
             for (int q = 0; q < kPre; q++) ld_slot(slots + (j & ~15) + q, scol[q], sval[q]);
         }
-        const double xin = ld_stream(b.x[src] + j);
+        double xin = (ALGO == ALG_AVERAGE || it == 0) ? ld_stream(b.x[src] + j) : b.xsum[j];
         const long long lk = ld_stream(b.lkey + j), uk = ld_stream(b.ukey + j);
         const double aux = (ALGO == ALG_AVERAGE) ? b.xsum[j] : ld_stream(b.xa + j);
         const bool st = SD && kk >= 0;
@@ -391,17 +409,13 @@ __global__ void __launch_bounds__(BS, 1536 / BS) k_primal(const Seg *__restrict_
         } else {
             for (int e = k0 + kPre; e < k1; e++) acc = fma(widen(ld_stream(v + e)), y[ld_stream(b.AT_ci + e)], acc);
         }
+        if (ALGO == ALG_HALPERN) xin = halpern_x(b, S, it, j, xin, aux);
         const double xv = clip_keys(fma(S->tau, acc, xin), lk, uk);
         if (ALGO == ALG_AVERAGE) {
             b.x[src ^ 1][j] = xv;
             b.xsum[j] = aux + xv;
         } else {
-            double w, w1;
-            halpern_weights(b, S, it, w, w1);
-            const double xb = fma(2.0, xv, -xin);
-            b.xsum[j] = xb;
-            b.x[src ^ 1][j] = fma(w, xb, w1 * aux);
-            if (keep) b.xret[j] = xv;
+            halpern_store(b, S, it, src, j, xin, xv, keep);
         }
     }
     if (!waited) { pdl_wait(); pdl_trigger(); }
