@@ -16,40 +16,75 @@
 //
 // Per iteration, evaluation included (30 / 300 / 1,441 buses of 24 periods): two
 // launches 8.05 / 8.25 / 9.4 us; this kernel with a grid-wide barrier after each
-// half 4.75 / 5.55 / 7.7 us; with tagged elements 3.4 / 4.1 / 5.1 us.  What is left
-// is the chain of one iteration: two stores and tagged loads through L2 (0.5 us
+// half 4.75 / 5.55 / 7.7 us; with tagged elements 3.4 / 4.1 / 4.9 us.  What is left
+// there is the chain of one iteration: two stores and tagged loads through L2 (0.5 us
 // each), the FP64 instructions of the longest row (up to nine entries, each waiting
-// for the one before), and the evaluation.
+// for the one before), and the evaluation.  Larger LPs are bound by the FP64 pipe:
+// 948 k rows and columns (3,000 buses of 48 periods) 14.1 us, of which the pipe needs
+// 10.2, and 1.9 M (6,049 buses) 27.1 us of which 20.4; row kernels 18.9 and 33.1.
+// They fit because entries that consecutive rows share are kept once and the rows'
+// constants are read from L2 (entries per row and constants kept: 474 k at most).
 #pragma once
 
 namespace uc {
 namespace dev {
 
 constexpr int kTileRows = 32;          // rows of a tile: one per lane
+
+// Threads of a CTA, and gathers in flight per row: what the registers hold without
+// spills, which live at L2's latency here (896 threads with 4 gathers: 29 us at 1.9 M
+// rows and columns against 27.1 with 3; 1,024 with 2: 27.7).  Few tiles: up to eight
+// warps.  Else 24 warps, or 28 where there are more than kBigTiles tiles per warp of the
+// 24 and the pipe's load counts rather than a row's latency: 632 k rows and columns (5.6
+// tiles) 10.1 us with 28, 10.35 with 24, 1.9 M 27.1 and 29.2; but 440 k without angles (4.0,
+// rows of up to 16 entries) 14.0 and 12.6.
+constexpr int kSmallThreads = 256, kSmallN = 8;
+constexpr int kMidThreads = 768, kMidN = 4;
+constexpr int kBigThreads = 896, kBigN = 3;
+constexpr int kBigTiles = 5;
 constexpr int kBlockMaxLps = 64;       // per-LP step data in shared memory
 constexpr int kBlockMaxEval = 1024;    // one LP: the weights of a block's iterations in shared memory
 
-// A tile: rows [r0, r0 + rows) of A^T or A; its entries in shared memory as
-// columns and values at q * 32 + lane, kmax per lane, beside its vectors.  A long
-// column (rows = 1, is_long) spreads its entries over the lanes in the same layout.
-struct __align__(16) BlockTile { int r0, rows, lp, aux, kmax, smem, is_long, pad; };
+// A tile: rows [r0, r0 + rows) of A^T or A.  In shared memory: the descriptor, the
+// rows' own vector (primal x-bar, dual y), then kmax entries per row as values, as
+// columns, and the rows' entry counts.  In the device layout consecutive rows are
+// mostly one constraint or variable of one entity in consecutive periods: where
+// entry q of row s of every group of 2^lg rows (lg 3 to 5) is (col_q + s, val_q), the
+// entries are kept once per group, entry q of group g at kmax g + q; else (lg 0) entry
+// q of lane l is at 32 q + l.  A uniform tile is grouped and all its rows have
+// kmax <= kUniform entries; a long column (one row) spreads its entries over the
+// lanes.
+enum TileKind : int { TILE_ANY = 0, TILE_LONG = 1, TILE_UNIFORM = 2 };
+struct __align__(16) BlockTile {
+    int r0;
+    unsigned info;   // see tile_info
+    int kmax, smem;
+};
+__host__ __device__ constexpr unsigned tile_info(int rows, int kind, int lg, bool primal, bool ineq, int lp) {
+    return (unsigned)rows | (unsigned)kind << 6 | (unsigned)lg << 8 | (unsigned)primal << 11 | (unsigned)ineq << 12 | (unsigned)lp << 13;
+}
+__host__ __device__ constexpr int tile_rows(unsigned info) { return info & 63; }
+__host__ __device__ constexpr int tile_kind(unsigned info) { return info >> 6 & 3; }
+__host__ __device__ constexpr int tile_lg(unsigned info) { return info >> 8 & 7; }
+__host__ __device__ constexpr bool tile_primal(unsigned info) { return info >> 11 & 1; }
+__host__ __device__ constexpr bool tile_ineq(unsigned info) { return info >> 12 & 1; }
+__host__ __device__ constexpr int tile_lp(unsigned info) { return info >> 13; }
+constexpr int kUniform = 4;
 // a warp's tiles: primal ones first
-struct BlockWarp { int first, primal, dual, pad; };
+struct BlockWarp { int first, count; };
 struct BlockPlan {
     const BlockTile *tiles;
     const BlockWarp *warps;       // by CTA, then warp
     const unsigned *seq;          // iterations of earlier launches (the evaluation adds this one's)
     ulonglong2 *xt, *yt;          // x-bar and y, tagged
     unsigned long long *stamp;    // kernel timing: the timed iteration's bounds on CTA 0 (or null)
-    int stamp_it, nlps, n_eval, head;   // head: bytes before the tiles' part of shared memory
-    int pad;
+    int stamp_it, nlps, n_eval, head;   // head: bytes before the warps' staged constants and the tiles
 };
 struct __align__(16) BlockLp { double tau, nsigma; int j, lim, pad[2]; };
 
-// descriptor, vectors (primal x-bar, x0, c, lower key, upper key; dual y, y0, q),
-// values, columns, entries per lane
-__host__ __device__ constexpr int tile_bytes(int kmax, bool primal) {
-    return (int)sizeof(BlockTile) + kTileRows * (kmax * 12 + (primal ? 40 : 24) + 4);
+constexpr int kStageBytes = 4 * kTileRows * 8;   // a tile's constants: primal c, x0 and the bounds' keys, dual q and y0
+__host__ __device__ constexpr int tile_bytes(int kmax, int lg) {
+    return (int)sizeof(BlockTile) + kTileRows * 8 + ((kTileRows >> lg) * (kmax * 12 + 4) + 15) / 16 * 16;
 }
 
 // A tagged element: two 64-bit words, each half of the double's bits below the
@@ -66,49 +101,65 @@ __device__ __forceinline__ ulonglong2 ld_tagged(const ulonglong2 *p) {
     return w;
 }
 
-// acc + (this lane's entries) . g, in order, N gathers in flight.  g: plain vector
-// (the block's start), or tagged and awaited.  Every wait ends: after four seconds
-// *stalled is set and the caller leaves.
-constexpr unsigned long long kBlockWaitNs = 4000000000ull;
-template <int N, bool TAGGED>
-__device__ __forceinline__ double tile_dot(double acc, const double *g, const ulonglong2 *gt, unsigned tag, const int *col,
-                                           const double *val, int kmax, int cnt, bool &stalled) {
+// Every wait ends: after so many polls (0.3 to 1 us each) *stalled is set and the
+// caller leaves.
+constexpr unsigned kBlockPolls = 1u << 22;
+
+// arrived() + (this lane's entries) . g, in order, N gathers in flight; entry q at
+// q * STEP, its column plus add; g tagged and awaited.  ALL: every lane has N entries.  arrived()
+// is called when the first words are there.
+template <int N, int STEP, bool ALL, typename F>
+__device__ __forceinline__ double tile_dot(const ulonglong2 *g, unsigned tag, const int *col, const double *val,
+                                           int add, int kmax, int cnt, bool &stalled, F &&arrived) {
+    double acc = 0.0;
+    g += add;
 #pragma unroll 1
-    for (int e = 0; e < kmax; e += N) {
-        double gv[N];
-        if (TAGGED) {
-            ulonglong2 w[N];
+    for (int e = 0; e < (ALL ? 1 : kmax); e += N) {
+        ulonglong2 w[N];
 #pragma unroll
-            for (int q = 0; q < N; q++) if (e + q < cnt) w[q] = ld_tagged(gt + col[(e + q) * kTileRows]);
-            unsigned long long t0 = 0;
-            for (unsigned n = 0;; n++) {
-                bool ready = true;
+        for (int q = 0; q < N; q++) if (ALL || e + q < cnt) w[q] = ld_tagged(g + col[(e + q) * STEP]);
+        for (unsigned n = 0;; n++) {
+            bool ready = true;
 #pragma unroll
-                for (int q = 0; q < N; q++)
-                    if (e + q < cnt && ((unsigned)(w[q].x >> 32) != tag || (unsigned)(w[q].y >> 32) != tag)) {
-                        ready = false;
-                        w[q] = ld_tagged(gt + col[(e + q) * kTileRows]);
-                    }
-                if (__all_sync(0xffffffffu, ready)) break;
-                if ((n & 255) == 255) {
-                    const unsigned long long t = global_ns();
-                    if (t0 == 0) t0 = t;
-                    if (__any_sync(0xffffffffu, t - t0 > kBlockWaitNs)) { stalled = true; return acc; }
+            for (int q = 0; q < N; q++)
+                if ((ALL || e + q < cnt) && ((unsigned)(w[q].x >> 32) != tag || (unsigned)(w[q].y >> 32) != tag)) {
+                    ready = false;
+                    w[q] = ld_tagged(g + col[(e + q) * STEP]);
                 }
-            }
-#pragma unroll
-            for (int q = 0; q < N; q++) gv[q] = __hiloint2double((int)(unsigned)w[q].y, (int)(unsigned)w[q].x);
-        } else {
-#pragma unroll
-            for (int q = 0; q < N; q++) if (e + q < cnt) gv[q] = g[col[(e + q) * kTileRows]];
+            if (__all_sync(0xffffffffu, ready)) break;
+            if (n > kBlockPolls) { stalled = true; return acc; }
         }
+        if (ALL || e == 0) acc = arrived();
 #pragma unroll
         for (int q = 0; q < N; q++) {
-            if (e + q >= kmax) break;
-            if (e + q < cnt) acc = fma(val[(e + q) * kTileRows], gv[q], acc);
+            if (!ALL && e + q >= kmax) break;
+            if (ALL || e + q < cnt)
+                acc = fma(val[(e + q) * STEP], __hiloint2double((int)(unsigned)w[q].y, (int)(unsigned)w[q].x), acc);
         }
     }
     return acc;
+}
+// the same from a plain vector (the block's start)
+__device__ __forceinline__ double plain_dot(double acc, const double *g, const int *col, const double *val, int step,
+                                            int add, int cnt) {
+#pragma unroll 4
+    for (int e = 0; e < cnt; e++) acc = fma(val[e * step], g[col[e * step] + add], acc);
+    return acc;
+}
+
+// asynchronous copy of eight bytes to shared memory
+__device__ __forceinline__ void copy8(double *dst, const void *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy8_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+__device__ __forceinline__ void stage_row(const Bufs &b, double *stage, bool primal, int r) {
+    copy8(stage, (primal ? b.c : b.q) + r);
+    copy8(stage + 32, (primal ? b.xa : b.ya) + r);
+    if (primal) {
+        copy8(stage + 64, b.lkey + r);
+        copy8(stage + 96, b.ukey + r);
+    }
 }
 
 __device__ __forceinline__ void block_weights(const Bufs &b, int jj, double &w, double &w1) {
@@ -122,14 +173,18 @@ __device__ __forceinline__ void block_weights(const Bufs &b, int jj, double &w, 
 }
 
 // Shared memory: the LPs' step data, ONE (a session of one LP): the weights
-// {w, 1 - w} of iteration it at it + 1, then the CTA's tiles.  A column keeps x-bar
+// {w, 1 - w} of iteration it at it + 1, then the CTA's tiles.  A row's constants come
+// from L1 or L2 each iteration, in flight with its gathers: into registers, or in
+// the largest CTAs (STAGED), which have none to spare, into kStageBytes of the warp's
+// (1.9 M rows and columns 27.1 us; loaded once the gathers are there 29.1).  A column keeps x-bar
 // (its x is w x-bar + (1 - w) x0, the Halpern step, computed when it is needed
 // next).  The last iteration of the block (or before the limit) writes what the
 // evaluation and the results read.
 template <typename VT, int NT, bool ONE>
 __global__ void __launch_bounds__(NT, 1) k_block(const __grid_constant__ BlockPlan P, const __grid_constant__ Bufs b) {
     extern __shared__ __align__(16) unsigned char blk_smem[];
-    constexpr int N = NT > 256 ? 4 : 8;   // gathers in flight per row: what the registers hold without spills
+    constexpr int N = NT > kMidThreads ? kBigN : NT > kSmallThreads ? kMidN : kSmallN;
+    constexpr bool STAGED = NT > kMidThreads;
     __shared__ int nit_;
     BlockLp *lps = reinterpret_cast<BlockLp *>(blk_smem);
     double2 *wt = reinterpret_cast<double2 *>(lps + P.nlps);
@@ -155,108 +210,144 @@ __global__ void __launch_bounds__(NT, 1) k_block(const __grid_constant__ BlockPl
             if (jj >= 0) block_weights(b, jj, w, w1);
             wt[t] = make_double2(w, w1);
         }
+    double *stage = reinterpret_cast<double *>(blk_smem + P.head + (threadIdx.x >> 5) * kStageBytes) + lane;   // STAGED
     // the warp's tiles into shared memory
     const BlockWarp wp = P.warps[blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)];
-    unsigned char *pool = blk_smem + P.head;
 #pragma unroll 1
-    for (int t = 0; t < wp.primal + wp.dual; t++) {
+    for (int t = 0; t < wp.count; t++) {
         const BlockTile T = P.tiles[wp.first + t];
-        const bool primal = t < wp.primal, ok = lane < T.rows;
-        if (lane == 0) *reinterpret_cast<BlockTile *>(pool + T.smem) = T;
-        double *vec = reinterpret_cast<double *>(pool + T.smem + sizeof(BlockTile));
-        double *val = vec + (primal ? 5 : 3) * kTileRows;
-        int *col = reinterpret_cast<int *>(val + T.kmax * kTileRows);
+        const bool primal = tile_primal(T.info), ok = lane < tile_rows(T.info), lng = tile_kind(T.info) == TILE_LONG;
+        unsigned char *here = blk_smem + T.smem;
+        if (lane == 0) *reinterpret_cast<BlockTile *>(here) = T;
+        double *z = reinterpret_cast<double *>(here + sizeof(BlockTile)), *val = z + kTileRows;
+        const int lg = tile_lg(T.info), width = kTileRows >> lg, at = lane >> lg;
+        int *col = reinterpret_cast<int *>(val + T.kmax * width);
         const int r = T.r0 + lane;
         const int *rp = primal ? b.AT_rp : b.A_rp, *ci = primal ? b.AT_ci : b.A_ci;
         const VT *v = static_cast<const VT *>(primal ? b.AT_v : b.A_v);
         int k0 = 0, k1 = 0, ks = 1;
-        if (T.is_long) { k0 = rp[T.r0] + lane; k1 = rp[T.r0 + 1]; ks = 32; }
+        if (lng) { k0 = rp[T.r0] + lane; k1 = rp[T.r0 + 1]; ks = 32; }
         else if (ok) { k0 = rp[r]; k1 = rp[r + 1]; }
-        for (int q = 0; q < T.kmax; q++) {
-            const int k = k0 + q * ks;
-            col[q * kTileRows + lane] = k < k1 ? ci[k] : 0;
-            val[q * kTileRows + lane] = k < k1 ? widen(v[k]) : 0.0;
+        if ((at << lg) == lane) {
+            const int first = lg ? at * T.kmax : lane, step = lg ? 1 : kTileRows;
+            for (int q = 0; q < T.kmax; q++) {
+                const int k = k0 + q * ks;
+                col[first + q * step] = k < k1 ? ci[k] : 0;
+                val[first + q * step] = k < k1 ? widen(v[k]) : 0.0;
+            }
+            col[T.kmax * width + at] = k1 > k0 ? (k1 - k0 + ks - 1) / ks : 0;
         }
-        col[T.kmax * kTileRows + lane] = k1 > k0 ? (k1 - k0 + ks - 1) / ks : 0;
-        if (ok && primal) {
-            vec[lane] = b.x[0][r];
-            vec[32 + lane] = b.xa[r];
-            vec[64 + lane] = b.c[r];
-            vec[96 + lane] = __longlong_as_double(b.lkey[r]);
-            vec[128 + lane] = __longlong_as_double(b.ukey[r]);
-        } else if (ok) {
-            vec[lane] = b.y[0][r];
-            vec[32 + lane] = b.ya[r];
-            vec[64 + lane] = b.q[r];
-        }
+        if (ok) z[lane] = primal ? b.x[0][r] : b.y[0][r];
     }
+    const unsigned tile0 = wp.count ? P.tiles[wp.first].smem : 0;   // a warp's tiles lie side by side
     __syncthreads();
     const int nit = nit_;
-    unsigned char *const tile0 = wp.primal + wp.dual ? pool + P.tiles[wp.first].smem : pool;   // a warp's tiles lie side by side
     const bool stamps = P.stamp && blockIdx.x == 0 && threadIdx.x == 0;
     const unsigned seq = *P.seq;
     bool stalled = false;
 #pragma unroll 1
     for (int it = 0; it < nit; it++) {
-        const int src = it & 1;
-        const unsigned tag = seq + (unsigned)it + 1;
         if (stamps && it == P.stamp_it) P.stamp[0] = global_ns();
         if (stamps && it == P.stamp_it + 1) P.stamp[1] = global_ns();
-        unsigned char *here = tile0;
+        unsigned here = tile0;
 #pragma unroll 1
-        for (int t = 0; t < wp.primal + wp.dual; t++) {
-            const int4 ta = *reinterpret_cast<const int4 *>(here), tb = *reinterpret_cast<const int4 *>(here + 16);
-            const int r = ta.x + lane, kmax = tb.x;
-            double *vec = reinterpret_cast<double *>(here + sizeof(BlockTile));
-            const bool ok = lane < ta.y, primal = t < wp.primal, lng = tb.z != 0;
-            const BlockLp &L = lps[ONE ? 0 : ta.z];
-            const bool keep = it == (ONE ? nit : L.lim) - 1;
-            here += tile_bytes(kmax, primal);
-            const double *val = vec + (primal ? 5 : 3) * kTileRows + lane;
-            const int *col = reinterpret_cast<const int *>(val - lane + kmax * kTileRows) + lane;
-            const int cnt = col[kmax * kTileRows];
-            if (!ONE && it >= L.lim) continue;
-            double acc = lng ? 0.0 : neg_bits(ok ? vec[64 + lane] : 0.0);
-            if (primal && it == 0) acc = tile_dot<N, false>(acc, b.y[0], nullptr, 0, col, val, kmax, cnt, stalled);
-            else acc = tile_dot<N, true>(acc, nullptr, primal ? P.yt : P.xt, primal ? tag - 1 : tag, col, val, kmax, cnt, stalled);
-            if (stalled) break;
-            if (primal) {
+        for (int t = 0; t < wp.count; t++) {
+            double acc;
+            const unsigned tile = here;
+            double anchor = 0.0;
+            long long lk = 0, uk = 0;
+            {
+                const BlockTile T = *reinterpret_cast<const BlockTile *>(blk_smem + tile);
+                const int r = T.r0 + lane, kmax = T.kmax, lg = tile_lg(T.info);
+                const bool ok = lane < tile_rows(T.info), primal = tile_primal(T.info), lng = tile_kind(T.info) == TILE_LONG;
+                here += tile_bytes(kmax, lg);
+                if (!ONE && it >= lps[tile_lp(T.info)].lim) continue;
+                // the lane's entries: its group's, and the offset in it (lanes without a row: of the first row)
+                const int mine = ok || lng ? lane : 0, at = mine >> lg, add = mine - (at << lg);
+                const double *val = reinterpret_cast<const double *>(blk_smem + tile + sizeof(BlockTile)) + kTileRows;
+                const int *col = reinterpret_cast<const int *>(val + (kmax << (5 - lg)));
+                const int cnt = ok || lng ? col[(kmax << (5 - lg)) + at] : 0;
+                val += lg ? at * kmax : at;
+                col += lg ? at * kmax : at;
+                // the rows' constants, in flight with the gathers
+                double c0 = 0.0;
+                if (STAGED) {
+                    if (ok) stage_row(b, stage, primal, r);
+                } else if (ok) {
+                    c0 = __ldg((primal ? b.c : b.q) + r);
+                    anchor = __ldg((primal ? b.xa : b.ya) + r);
+                    if (NT <= kSmallThreads && primal) { lk = __ldg(b.lkey + r); uk = __ldg(b.ukey + r); }
+                }
+                auto arrived = [&] {
+                    if (STAGED) {
+                        copy8_wait();
+                        if (ok) c0 = *stage;
+                    }
+                    return lng ? 0.0 : neg_bits(c0);
+                };
+                const ulonglong2 *gt = primal ? P.yt : P.xt;
+                const unsigned want = seq + (unsigned)it + (primal ? 0u : 1u);
+                if (primal && it == 0) {
+                    acc = plain_dot(arrived(), b.y[0], col, val, lg ? 1 : kTileRows, add, cnt);
+                } else if (tile_kind(T.info) == TILE_UNIFORM) {
+                    if (kmax == 3) acc = tile_dot<3, 1, true>(gt, want, col, val, add, 3, 3, stalled, arrived);
+                    else if (kmax == 2) acc = tile_dot<2, 1, true>(gt, want, col, val, add, 2, 2, stalled, arrived);
+                    else if (kmax == 1) acc = tile_dot<1, 1, true>(gt, want, col, val, add, 1, 1, stalled, arrived);
+                    else if (kUniform == 4) acc = tile_dot<4, 1, true>(gt, want, col, val, add, 4, 4, stalled, arrived);
+                } else if (lg) acc = tile_dot<N, 1, false>(gt, want, col, val, add, kmax, cnt, stalled, arrived);
+                else acc = tile_dot<N, kTileRows, false>(gt, want, col, val, 0, kmax, cnt, stalled, arrived);
+                if (kmax == 0) acc = arrived();
+                if (stalled) break;
                 if (lng) {
 #pragma unroll
                     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-                    acc = neg_bits(vec[64]) + acc;
+                    acc = neg_bits(__shfl_sync(0xffffffffu, c0, 0)) + acc;
                 }
-                if (ok) {
-                    double x = vec[lane];
-                    const double x0 = vec[32 + lane];
-                    double2 w = make_double2(0.0, 0.0);
-                    if (it > 0) {
-                        if (ONE) w = wt[it];
-                        else block_weights(b, L.j + it - 1, w.x, w.y);
-                        x = fma(w.x, x, w.y * x0);
-                    }
-                    const double xv = clip_keys(fma(L.tau, acc, x), __double_as_longlong(vec[96 + lane]),
-                                                __double_as_longlong(vec[128 + lane]));
-                    const double xr = fma(2.0, xv, -x);
-                    st_tagged(P.xt + r, xr, tag);
-                    vec[lane] = xr;
-                    if (keep) {
-                        block_weights(b, L.j + it, w.x, w.y);
-                        b.x[src][r] = x;
-                        b.x[src ^ 1][r] = fma(w.x, xr, w.y * x0);
-                        b.xret[r] = xv;
-                    }
+            }
+            // the descriptor again: from shared memory, not kept in registers meanwhile
+            const int2 d = *reinterpret_cast<const int2 *>(blk_smem + tile);
+            const int r = d.x + lane, src = it & 1;
+            const unsigned tag = seq + (unsigned)it + 1;
+            double *z = reinterpret_cast<double *>(blk_smem + tile + sizeof(BlockTile)) + lane;
+            const BlockLp &L = lps[ONE ? 0 : tile_lp(d.y)];
+            const bool keep = it == (ONE ? nit : L.lim) - 1;
+            if (lane >= tile_rows(d.y)) continue;
+            if (STAGED) anchor = stage[32];
+            if (tile_primal(d.y)) {
+                if (STAGED) {
+                    lk = __double_as_longlong(stage[64]);
+                    uk = __double_as_longlong(stage[96]);
+                } else if (NT > kSmallThreads) {
+                    lk = __ldg(b.lkey + r);
+                    uk = __ldg(b.ukey + r);
                 }
-            } else if (ok) {
-                const double y = vec[lane];
+                double x = *z;
+                double2 w = make_double2(0.0, 0.0);
+                if (it > 0) {
+                    if (ONE) w = wt[it];
+                    else block_weights(b, L.j + it - 1, w.x, w.y);
+                    x = fma(w.x, x, w.y * anchor);
+                }
+                const double xv = clip_keys(fma(L.tau, acc, x), lk, uk);
+                const double xr = fma(2.0, xv, -x);
+                st_tagged(P.xt + r, xr, tag);
+                *z = xr;
+                if (keep) {
+                    block_weights(b, L.j + it, w.x, w.y);
+                    b.x[src][r] = x;
+                    b.x[src ^ 1][r] = fma(w.x, xr, w.y * anchor);
+                    b.xret[r] = xv;
+                }
+            } else {
+                const double y = *z;
                 double yv = fma(L.nsigma, acc, y);
-                if (r >= ta.w) yv = nonneg(yv);
+                if (tile_ineq(d.y)) yv = nonneg(yv);
                 double2 w;
                 if (ONE) w = wt[it + 1];
                 else block_weights(b, L.j + it, w.x, w.y);
-                const double yn = fma(w.x, fma(2.0, yv, -y), w.y * vec[32 + lane]);
+                const double yn = fma(w.x, fma(2.0, yv, -y), w.y * anchor);
                 st_tagged(P.yt + r, yn, tag);
-                vec[lane] = yn;
+                *z = yn;
                 if (keep) {
                     b.y[src][r] = y;
                     b.y[src ^ 1][r] = yn;

@@ -2317,8 +2317,9 @@ static void launch_adaptive_norm(uc_session &X, cudaStream_t s) {
 using BlockKernel = void (*)(BlockPlan, Bufs);
 template <typename VT>
 static BlockKernel block_kernel_vt(int threads, bool one) {
-    if (threads <= 256) return one ? k_block<VT, 256, true> : k_block<VT, 256, false>;
-    return one ? k_block<VT, 1024, true> : k_block<VT, 1024, false>;
+    if (threads <= kSmallThreads) return one ? k_block<VT, kSmallThreads, true> : k_block<VT, kSmallThreads, false>;
+    if (threads <= kMidThreads) return one ? k_block<VT, kMidThreads, true> : k_block<VT, kMidThreads, false>;
+    return one ? k_block<VT, kBigThreads, true> : k_block<VT, kBigThreads, false>;
 }
 static BlockKernel block_kernel(const uc_session &X, int threads) {
     return X.vb == 32 ? block_kernel_vt<float>(threads, X.k == 1) : block_kernel_vt<double>(threads, X.k == 1);
@@ -2493,6 +2494,26 @@ static void build_tables(const uc_session &X, const std::vector<char> &mask, std
     sa.insert(sa.end(), sd.begin(), sd.end());
 }
 
+// Largest lg in 5, 4, 3 such that entry q of row s of every group of 2^lg of the
+// rows [a, b) of M (the last may be short) is (col_q + s, val_q), values as stored;
+// 0 if there is none.  v32: the FP32 values, if M is stored so.
+static int tile_group(const Csr &M, const std::vector<float> &v32, int a, int b) {
+    int lg = 5;
+    for (int r = a + 1; r < b; r++) {
+        while (lg >= 3) {
+            const int s = (r - a) & ((1 << lg) - 1), e0 = M.rowptr[r - s], e = M.rowptr[r], k = M.rowptr[r + 1] - e;
+            bool same = M.rowptr[r - s + 1] - e0 == k;
+            for (int q = 0; s > 0 && same && q < k; q++)
+                same = M.colidx[e + q] == M.colidx[e0 + q] + s &&
+                       (v32.empty() ? M.val[e + q] == M.val[e0 + q] : v32[e + q] == v32[e0 + q]);
+            if (same) break;
+            lg--;
+        }
+        if (lg < 3) return 0;
+    }
+    return lg;
+}
+
 // Tiles of the resident block kernel for the LPs in `mask`, dealt to the warps of
 // at most one CTA per SM: primal tiles, longest rows first, to the warps in turn
 // over the CTAs, dual tiles in turn from the last warp back, so that a warp has
@@ -2510,58 +2531,71 @@ static void plan_block(uc_session &X, const std::vector<char> &mask, std::vector
         if (!mask[i]) continue;
         const PsData &v = *X.Pd[i];
         const int n = v.n(), m = v.m(), nl = v.long_cols, m_eq = X.m_eq[i];
-        auto cut = [&](const Csr &M, int a, int b, int64_t base, int aux, bool primal) {
+        auto cut = [&](const Csr &M, int a, int b, int64_t base, bool primal, bool ineq) {
             for (int s = a; s < b; s += kTileRows) {
                 const int e = std::min(b, s + kTileRows);
-                int kmax = 0;
-                for (int r = s; r < e; r++) kmax = std::max(kmax, M.rowptr[r + 1] - M.rowptr[r]);
-                t[primal].push_back(BlockTile{(int)(base + s), e - s, i, aux, kmax, 0, 0, 0});
-                bytes += tile_bytes(kmax, primal);
+                int kmax = 0, kmin = INT_MAX;
+                for (int r = s; r < e; r++) {
+                    kmax = std::max(kmax, M.rowptr[r + 1] - M.rowptr[r]);
+                    kmin = std::min(kmin, M.rowptr[r + 1] - M.rowptr[r]);
+                }
+                const int lg = tile_group(M, primal ? v.AT_val32 : v.A_val32, s, e);
+                const int kind = lg && kmin == kmax && kmax >= 1 && kmax <= kUniform ? TILE_UNIFORM : TILE_ANY;
+                t[primal].push_back(BlockTile{(int)(base + s), tile_info(e - s, kind, lg, primal, ineq, i), kmax, 0});
+                bytes += tile_bytes(kmax, lg);
             }
         };
-        cut(v.AT, 0, n - nl, X.coff[i], 0, true);
+        cut(v.AT, 0, n - nl, X.coff[i], true, false);
         for (int j = n - nl; j < n; j++) {
             const int kmax = (v.AT.rowptr[j + 1] - v.AT.rowptr[j] + 31) / 32;
-            t[1].push_back(BlockTile{(int)(X.coff[i] + j), 1, i, 0, kmax, 0, 1, 0});
-            bytes += tile_bytes(kmax, true);
+            t[1].push_back(BlockTile{(int)(X.coff[i] + j), tile_info(1, TILE_LONG, 0, true, false, i), kmax, 0});
+            bytes += tile_bytes(kmax, 0);
         }
-        cut(v.A, 0, m, X.roff[i], (int)X.roff[i] + m_eq, false);
+        cut(v.A, 0, m_eq, X.roff[i], false, false);
+        cut(v.A, m_eq, m, X.roff[i], false, true);
         if (bytes > (int64_t)X.sms * X.blk_smem_max) return;
     }
     const int64_t np = t[1].size(), nd = t[0].size();
     if (np == 0 || nd == 0) return;
     const int nc = (int)std::min<int64_t>(X.sms, std::max(np, nd));
-    const int W = (int)std::min<int64_t>(32, (np + nd + nc - 1) / nc);
+    const bool big = np + nd > (int64_t)kBigTiles * nc * (kMidThreads / 32);
+    const int W = (int)std::min<int64_t>((big ? kBigThreads : kMidThreads) / 32, (np + nd + nc - 1) / nc);
     const int64_t S = (int64_t)nc * W;
     std::vector<std::vector<const BlockTile *>> mine[2];
     for (int ph = 0; ph < 2; ph++) {
         mine[ph].resize(S);
-        std::stable_sort(t[ph].begin(), t[ph].end(), [](const BlockTile &a, const BlockTile &b) { return a.kmax > b.kmax; });
+        std::stable_sort(t[ph].begin(), t[ph].end(), [](const BlockTile &a, const BlockTile &b) {
+            return a.kmax != b.kmax ? a.kmax > b.kmax : tile_lg(a.info) < tile_lg(b.info);
+        });
         for (int64_t i = 0; i < (int64_t)t[ph].size(); i++) mine[ph][ph ? i % S : S - 1 - i % S].push_back(&t[ph][i]);
     }
-    const int head = block_head(X);
-    int most = 0;
-    for (int c = 0; c < nc; c++) {
-        int64_t at = 0;
+    for (int c = 0; c < nc; c++)
         for (int w = 0; w < W; w++) {
             const int64_t slot = (int64_t)w * nc + c;
-            warps.push_back(BlockWarp{(int)tiles.size(), (int)mine[1][slot].size(), (int)mine[0][slot].size(), 0});
+            warps.push_back(BlockWarp{(int)tiles.size(), (int)(mine[1][slot].size() + mine[0][slot].size())});
             for (int ph = 1; ph >= 0; ph--)
-                for (const BlockTile *p : mine[ph][slot]) {
-                    tiles.push_back(*p);
-                    tiles.back().smem = (int)at;
-                    at += tile_bytes(p->kmax, ph == 1);
-                    if (head + at > X.blk_smem_max) return;
-                }
+                for (const BlockTile *p : mine[ph][slot]) tiles.push_back(*p);
         }
-        most = std::max(most, (int)at);
+    const int head = block_head(X);
+    int64_t most = 0;
+    for (int c = 0; c < nc; c++) {
+        int64_t at = head + (big ? W * kStageBytes : 0);
+        for (int w = 0; w < W; w++) {
+            const BlockWarp &wp = warps[(size_t)c * W + w];
+            for (int q = wp.first; q < wp.first + wp.count; q++) {
+                tiles[q].smem = (int)at;
+                at += tile_bytes(tiles[q].kmax, tile_lg(tiles[q].info));
+            }
+        }
+        most = std::max(most, at);
     }
+    if (most > X.blk_smem_max) return;
     X.plan.head = head;
     X.plan.nlps = X.k;
     X.plan.n_eval = X.o.n_eval;
     X.blk_ctas = nc;
     X.blk_threads = 32 * W;
-    X.blk_smem = head + most;
+    X.blk_smem = (int)most;
     X.block = true;
 }
 
@@ -2819,7 +2853,7 @@ static int session_create(const PsData *const *Pp, const std::shared_ptr<const P
         X->block_able = coop && o.spmv_kernel == 0 && X->algo == ALG_HALPERN && X->K == 1 && k <= kBlockMaxLps &&
                         o.n_eval <= kBlockMaxEval;
         if (X->block_able)
-            for (int nt : {256, 1024})
+            for (int nt : {kSmallThreads, kMidThreads, kBigThreads})
                 UC_CUDA(cudaFuncSetAttribute(block_kernel(*X, nt), cudaFuncAttributeMaxDynamicSharedMemorySize, X->blk_smem_max));
         plan_block(*X, all, tiles, warps);
         if (k == 1 && !X->block) X->block_able = false;   // no subset of its LPs fits either
@@ -2853,11 +2887,11 @@ static int session_create(const PsData *const *Pp, const std::shared_ptr<const P
     L.inv_Dc = take(N * 8); L.lkey = take(N * 8); L.ukey = take(N * 8);
     L.q = take(M * 8); L.Dr = take(M * 8); L.inv_Dr = take(M * 8);
     L.x_init = take(N * 8); L.y_init = take(M * 8); L.S_init = take(sizeof(Scalars) * k);
-    {   // tables for any subset of the LPs: a tile per 32 rows or columns begun, or per long column
+    {   // tables for any subset of the LPs: a tile per 32 rows or columns begun (rows: of either kind), or per long column
         int64_t nt = 0;
         for (int i = 0; i < k && X->block_able; i++) {
             const PsData &p = *X->Pd[i];
-            nt += (p.n() + kTileRows - 1) / kTileRows + (p.m() + kTileRows - 1) / kTileRows + p.long_cols;
+            nt += (p.n() + kTileRows - 1) / kTileRows + (p.m() + kTileRows - 1) / kTileRows + 1 + p.long_cols;
         }
         L.tiles = take(sizeof(BlockTile) * nt);
         L.warps = take(X->block_able ? sizeof(BlockWarp) * 32 * X->sms : 0);

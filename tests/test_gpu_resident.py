@@ -50,6 +50,16 @@ def test_resident_kernel_equals_row_kernels(B, buses, periods, units, value_bits
     _same(B, a, B.uc_solve(ps, tol=0.0, max_iter=100, n_eval=2, use_graph=False)[0], ps)
 
 
+# shared entries in groups of 8, 16 and 32 rows, in none (periods of 10 and 31), and the
+# largest CTAs (2,000 buses of 48 periods: more than five tiles per warp)
+@pytest.mark.parametrize("buses,periods,units", [(70, 8, 9), (60, 10, 9), (50, 16, 6), (45, 32, 6), (64, 31, 8), (2000, 48, 240)])
+@pytest.mark.parametrize("value_bits", [64, 32])
+def test_resident_kernel_with_shared_entries(B, buses, periods, units, value_bits):
+    ps = B.uc_presolve(B.uc_build_lp(_grid(buses, buses, periods, units)), value_bits=value_bits, power_max_iter=20)
+    for budget in (1, 64, 130):
+        _same(B, B.uc_solve(ps, tol=0.0, max_iter=budget, spmv_kernel=1)[0], B.uc_solve(ps, tol=0.0, max_iter=budget)[0], ps)
+
+
 def test_resident_kernel_with_long_columns(B):
     ps = B.uc_presolve(B.uc_build_lp(_grid(3, 500, 24, 60)), eliminate_angles=1, power_max_iter=20)
     for budget in (1, 64, 150):
