@@ -20,10 +20,12 @@
 // there is the chain of one iteration: two stores and tagged loads through L2 (0.5 us
 // each), the FP64 instructions of the longest row (up to nine entries, each waiting
 // for the one before), and the evaluation.  Larger LPs are bound by the FP64 pipe:
-// 948 k rows and columns (3,000 buses of 48 periods) 14.1 us, of which the pipe needs
-// 10.2, and 1.9 M (6,049 buses) 27.1 us of which 20.4; row kernels 18.9 and 33.1.
-// They fit because entries that consecutive rows share are kept once and the rows'
-// constants are read from L2 (entries per row and constants kept: 474 k at most).
+// 948 k rows and columns (3,000 buses of 48 periods) 14.0 us, of which the pipe needs
+// 10.2, and 1.9 M (6,049 buses) 26.9 us of which 20.4; row kernels 18.9 and 33.1.
+// They fit because a run's entries are kept once and the rows' constants are read
+// from L2: 1.9 M take 164 KB per SM and 2.5 M 205 KB (entries per row and constants
+// kept: 474 k at most; entries shared by aligned groups of 8 to 32 rows: 215 KB at
+// 1.9 M, and eight LPs of 24 and 48 periods with as many rows did not fit).
 #pragma once
 
 namespace uc {
@@ -32,12 +34,13 @@ namespace dev {
 constexpr int kTileRows = 32;          // rows of a tile: one per lane
 
 // Threads of a CTA, and gathers in flight per row: what the registers hold without
-// spills, which live at L2's latency here (896 threads with 4 gathers: 29 us at 1.9 M
-// rows and columns against 27.1 with 3; 1,024 with 2: 27.7).  Few tiles: up to eight
-// warps.  Else 24 warps, or 28 where there are more than kBigTiles tiles per warp of the
-// 24 and the pipe's load counts rather than a row's latency: 632 k rows and columns (5.6
-// tiles) 10.1 us with 28, 10.35 with 24, 1.9 M 27.1 and 29.2; but 440 k without angles (4.0,
-// rows of up to 16 entries) 14.0 and 12.6.
+// spills, which live at L2's latency here.  Few tiles: up to eight warps.  Else 24
+// warps, or 28 where there are more than kBigTiles tiles per warp of the 24 and the
+// pipe's load counts rather than a row's latency: 632 k rows and columns (5.6 tiles)
+// 10.1 us with 28, 10.35 with 24, 1.9 M 27.1 and 29.2; but 440 k without angles (4.0, rows
+// of up to 16 entries) 14.0 and 12.6.  Gathers with 24 warps, 4 / 5 / 6: 7.9 / 7.4 / 8.4
+// us at 55 k without angles, 12.7 / 13.1 / 13.2 at 440 k.  32 warps with 2: 26.9 us
+// at 1.9 M, as 28 with 3.
 constexpr int kSmallThreads = 256, kSmallN = 8;
 constexpr int kMidThreads = 768, kMidN = 4;
 constexpr int kBigThreads = 896, kBigN = 3;
@@ -45,30 +48,36 @@ constexpr int kBigTiles = 5;
 constexpr int kBlockMaxLps = 64;       // per-LP step data in shared memory
 constexpr int kBlockMaxEval = 1024;    // one LP: the weights of a block's iterations in shared memory
 
-// A tile: rows [r0, r0 + rows) of A^T or A.  In shared memory: the descriptor, the
-// rows' own vector (primal x-bar, dual y), then kmax entries per row as values, as
-// columns, and the rows' entry counts.  In the device layout consecutive rows are
-// mostly one constraint or variable of one entity in consecutive periods: where
-// entry q of row s of every group of 2^lg rows (lg 3 to 5) is (col_q + s, val_q), the
-// entries are kept once per group, entry q of group g at kmax g + q; else (lg 0) entry
-// q of lane l is at 32 q + l.  A uniform tile is grouped and all its rows have
-// kmax <= kUniform entries; a long column (one row) spreads its entries over the
-// lanes.
+// A tile: rows [r0, r0 + rows) of A^T or A.  In shared memory: the descriptor's
+// first 16 bytes, the rows' own vector (primal x-bar, dual y), then the entries as
+// values, as columns, and their counts, once per run.  A run is consecutive rows
+// whose entry q is (col_q + s, val_q) for the s-th row, in the device layout mostly one
+// constraint or variable of one entity over the periods; bit l of runs is set where a
+// run begins at lane l.  Entry q of run g is at g stride + q.  A uniform tile's rows all
+// have kmax <= kUniform entries; a long column (one row) spreads its entries over the
+// lanes, a run each.
 enum TileKind : int { TILE_ANY = 0, TILE_LONG = 1, TILE_UNIFORM = 2 };
 struct __align__(16) BlockTile {
     int r0;
     unsigned info;   // see tile_info
-    int kmax, smem;
+    int kmax;
+    unsigned runs;
+    int smem, pad[3];
 };
-__host__ __device__ constexpr unsigned tile_info(int rows, int kind, int lg, bool primal, bool ineq, int lp) {
-    return (unsigned)rows | (unsigned)kind << 6 | (unsigned)lg << 8 | (unsigned)primal << 11 | (unsigned)ineq << 12 | (unsigned)lp << 13;
+constexpr int kTileHead = 16;
+__host__ __device__ constexpr unsigned tile_info(int rows, int kind, bool primal, bool ineq, int lp) {
+    return (unsigned)rows | (unsigned)kind << 6 | (unsigned)primal << 8 | (unsigned)ineq << 9 | (unsigned)lp << 10;
 }
 __host__ __device__ constexpr int tile_rows(unsigned info) { return info & 63; }
 __host__ __device__ constexpr int tile_kind(unsigned info) { return info >> 6 & 3; }
-__host__ __device__ constexpr int tile_lg(unsigned info) { return info >> 8 & 7; }
-__host__ __device__ constexpr bool tile_primal(unsigned info) { return info >> 11 & 1; }
-__host__ __device__ constexpr bool tile_ineq(unsigned info) { return info >> 12 & 1; }
-__host__ __device__ constexpr int tile_lp(unsigned info) { return info >> 13; }
+__host__ __device__ constexpr bool tile_primal(unsigned info) { return info >> 8 & 1; }
+__host__ __device__ constexpr bool tile_ineq(unsigned info) { return info >> 9 & 1; }
+__host__ __device__ constexpr int tile_lp(unsigned info) { return info >> 10; }
+// odd where many lanes read a run of their own: no bank is hit twice
+__host__ __device__ constexpr int tile_stride(int kmax, int runs) { return runs > 8 ? kmax | 1 : kmax; }
+__host__ __device__ constexpr int tile_bytes(int stride, int runs) {
+    return kTileHead + kTileRows * 8 + (runs * (stride * 12 + 4) + 15) / 16 * 16;
+}
 constexpr int kUniform = 4;
 // a warp's tiles: primal ones first
 struct BlockWarp { int first, count; };
@@ -83,9 +92,6 @@ struct BlockPlan {
 struct __align__(16) BlockLp { double tau, nsigma; int j, lim, pad[2]; };
 
 constexpr int kStageBytes = 4 * kTileRows * 8;   // a tile's constants: primal c, x0 and the bounds' keys, dual q and y0
-__host__ __device__ constexpr int tile_bytes(int kmax, int lg) {
-    return (int)sizeof(BlockTile) + kTileRows * 8 + ((kTileRows >> lg) * (kmax * 12 + 4) + 15) / 16 * 16;
-}
 
 // A tagged element: two 64-bit words, each half of the double's bits below the
 // tag.  A 64-bit access is never torn, so a word with the right tag has the right
@@ -106,9 +112,9 @@ __device__ __forceinline__ ulonglong2 ld_tagged(const ulonglong2 *p) {
 constexpr unsigned kBlockPolls = 1u << 22;
 
 // arrived() + (this lane's entries) . g, in order, N gathers in flight; entry q at
-// q * STEP, its column plus add; g tagged and awaited.  ALL: every lane has N entries.  arrived()
+// q, its column plus add; g tagged and awaited.  ALL: every lane has N entries.  arrived()
 // is called when the first words are there.
-template <int N, int STEP, bool ALL, typename F>
+template <int N, bool ALL, typename F>
 __device__ __forceinline__ double tile_dot(const ulonglong2 *g, unsigned tag, const int *col, const double *val,
                                            int add, int kmax, int cnt, bool &stalled, F &&arrived) {
     double acc = 0.0;
@@ -117,14 +123,14 @@ __device__ __forceinline__ double tile_dot(const ulonglong2 *g, unsigned tag, co
     for (int e = 0; e < (ALL ? 1 : kmax); e += N) {
         ulonglong2 w[N];
 #pragma unroll
-        for (int q = 0; q < N; q++) if (ALL || e + q < cnt) w[q] = ld_tagged(g + col[(e + q) * STEP]);
+        for (int q = 0; q < N; q++) if (ALL || e + q < cnt) w[q] = ld_tagged(g + col[e + q]);
         for (unsigned n = 0;; n++) {
             bool ready = true;
 #pragma unroll
             for (int q = 0; q < N; q++)
                 if ((ALL || e + q < cnt) && ((unsigned)(w[q].x >> 32) != tag || (unsigned)(w[q].y >> 32) != tag)) {
                     ready = false;
-                    w[q] = ld_tagged(g + col[(e + q) * STEP]);
+                    w[q] = ld_tagged(g + col[e + q]);
                 }
             if (__all_sync(0xffffffffu, ready)) break;
             if (n > kBlockPolls) { stalled = true; return acc; }
@@ -134,16 +140,15 @@ __device__ __forceinline__ double tile_dot(const ulonglong2 *g, unsigned tag, co
         for (int q = 0; q < N; q++) {
             if (!ALL && e + q >= kmax) break;
             if (ALL || e + q < cnt)
-                acc = fma(val[(e + q) * STEP], __hiloint2double((int)(unsigned)w[q].y, (int)(unsigned)w[q].x), acc);
+                acc = fma(val[e + q], __hiloint2double((int)(unsigned)w[q].y, (int)(unsigned)w[q].x), acc);
         }
     }
     return acc;
 }
 // the same from a plain vector (the block's start)
-__device__ __forceinline__ double plain_dot(double acc, const double *g, const int *col, const double *val, int step,
-                                            int add, int cnt) {
+__device__ __forceinline__ double plain_dot(double acc, const double *g, const int *col, const double *val, int add, int cnt) {
 #pragma unroll 4
-    for (int e = 0; e < cnt; e++) acc = fma(val[e * step], g[col[e * step] + add], acc);
+    for (int e = 0; e < cnt; e++) acc = fma(val[e], g[col[e] + add], acc);
     return acc;
 }
 
@@ -218,24 +223,24 @@ __global__ void __launch_bounds__(NT, 1) k_block(const __grid_constant__ BlockPl
         const BlockTile T = P.tiles[wp.first + t];
         const bool primal = tile_primal(T.info), ok = lane < tile_rows(T.info), lng = tile_kind(T.info) == TILE_LONG;
         unsigned char *here = blk_smem + T.smem;
-        if (lane == 0) *reinterpret_cast<BlockTile *>(here) = T;
-        double *z = reinterpret_cast<double *>(here + sizeof(BlockTile)), *val = z + kTileRows;
-        const int lg = tile_lg(T.info), width = kTileRows >> lg, at = lane >> lg;
-        int *col = reinterpret_cast<int *>(val + T.kmax * width);
+        if (lane == 0) *reinterpret_cast<int4 *>(here) = make_int4(T.r0, T.info, T.kmax, T.runs);
+        double *z = reinterpret_cast<double *>(here + kTileHead), *val = z + kTileRows;
+        const int runs = __popc(T.runs), stride = tile_stride(T.kmax, runs);
+        const int at = __popc(T.runs & ((2u << lane) - 1)) - 1;
+        int *col = reinterpret_cast<int *>(val + runs * stride);
         const int r = T.r0 + lane;
         const int *rp = primal ? b.AT_rp : b.A_rp, *ci = primal ? b.AT_ci : b.A_ci;
         const VT *v = static_cast<const VT *>(primal ? b.AT_v : b.A_v);
         int k0 = 0, k1 = 0, ks = 1;
         if (lng) { k0 = rp[T.r0] + lane; k1 = rp[T.r0 + 1]; ks = 32; }
         else if (ok) { k0 = rp[r]; k1 = rp[r + 1]; }
-        if ((at << lg) == lane) {
-            const int first = lg ? at * T.kmax : lane, step = lg ? 1 : kTileRows;
+        if (T.runs >> lane & 1) {
             for (int q = 0; q < T.kmax; q++) {
                 const int k = k0 + q * ks;
-                col[first + q * step] = k < k1 ? ci[k] : 0;
-                val[first + q * step] = k < k1 ? widen(v[k]) : 0.0;
+                col[at * stride + q] = k < k1 ? ci[k] : 0;
+                val[at * stride + q] = k < k1 ? widen(v[k]) : 0.0;
             }
-            col[T.kmax * width + at] = k1 > k0 ? (k1 - k0 + ks - 1) / ks : 0;
+            col[runs * stride + at] = k1 > k0 ? (k1 - k0 + ks - 1) / ks : 0;
         }
         if (ok) z[lane] = primal ? b.x[0][r] : b.y[0][r];
     }
@@ -257,18 +262,20 @@ __global__ void __launch_bounds__(NT, 1) k_block(const __grid_constant__ BlockPl
             double anchor = 0.0;
             long long lk = 0, uk = 0;
             {
-                const BlockTile T = *reinterpret_cast<const BlockTile *>(blk_smem + tile);
-                const int r = T.r0 + lane, kmax = T.kmax, lg = tile_lg(T.info);
-                const bool ok = lane < tile_rows(T.info), primal = tile_primal(T.info), lng = tile_kind(T.info) == TILE_LONG;
-                here += tile_bytes(kmax, lg);
-                if (!ONE && it >= lps[tile_lp(T.info)].lim) continue;
-                // the lane's entries: its group's, and the offset in it (lanes without a row: of the first row)
-                const int mine = ok || lng ? lane : 0, at = mine >> lg, add = mine - (at << lg);
-                const double *val = reinterpret_cast<const double *>(blk_smem + tile + sizeof(BlockTile)) + kTileRows;
-                const int *col = reinterpret_cast<const int *>(val + (kmax << (5 - lg)));
-                const int cnt = ok || lng ? col[(kmax << (5 - lg)) + at] : 0;
-                val += lg ? at * kmax : at;
-                col += lg ? at * kmax : at;
+                const int4 T = *reinterpret_cast<const int4 *>(blk_smem + tile);
+                const int r = T.x + lane, kmax = T.z, runs = __popc(T.w), stride = tile_stride(kmax, runs);
+                const bool ok = lane < tile_rows(T.y), primal = tile_primal(T.y), lng = tile_kind(T.y) == TILE_LONG;
+                here += tile_bytes(stride, runs);
+                if (!ONE && it >= lps[tile_lp(T.y)].lim) continue;
+                // the lane's run and its row in it (lanes without a row: the first)
+                const int mine = ok || lng ? lane : 0;
+                const unsigned upto = (unsigned)T.w & ((2u << mine) - 1);
+                const int at = __popc(upto) - 1, add = mine - (31 - __clz(upto));
+                const double *val = reinterpret_cast<const double *>(blk_smem + tile + kTileHead) + kTileRows;
+                const int *col = reinterpret_cast<const int *>(val + runs * stride);
+                const int cnt = ok || lng ? col[runs * stride + at] : 0;
+                val += at * stride;
+                col += at * stride;
                 // the rows' constants, in flight with the gathers
                 double c0 = 0.0;
                 if (STAGED) {
@@ -288,14 +295,13 @@ __global__ void __launch_bounds__(NT, 1) k_block(const __grid_constant__ BlockPl
                 const ulonglong2 *gt = primal ? P.yt : P.xt;
                 const unsigned want = seq + (unsigned)it + (primal ? 0u : 1u);
                 if (primal && it == 0) {
-                    acc = plain_dot(arrived(), b.y[0], col, val, lg ? 1 : kTileRows, add, cnt);
-                } else if (tile_kind(T.info) == TILE_UNIFORM) {
-                    if (kmax == 3) acc = tile_dot<3, 1, true>(gt, want, col, val, add, 3, 3, stalled, arrived);
-                    else if (kmax == 2) acc = tile_dot<2, 1, true>(gt, want, col, val, add, 2, 2, stalled, arrived);
-                    else if (kmax == 1) acc = tile_dot<1, 1, true>(gt, want, col, val, add, 1, 1, stalled, arrived);
-                    else if (kUniform == 4) acc = tile_dot<4, 1, true>(gt, want, col, val, add, 4, 4, stalled, arrived);
-                } else if (lg) acc = tile_dot<N, 1, false>(gt, want, col, val, add, kmax, cnt, stalled, arrived);
-                else acc = tile_dot<N, kTileRows, false>(gt, want, col, val, 0, kmax, cnt, stalled, arrived);
+                    acc = plain_dot(arrived(), b.y[0], col, val, add, cnt);
+                } else if (tile_kind(T.y) == TILE_UNIFORM) {
+                    if (kmax == 3) acc = tile_dot<3, true>(gt, want, col, val, add, 3, 3, stalled, arrived);
+                    else if (kmax == 2) acc = tile_dot<2, true>(gt, want, col, val, add, 2, 2, stalled, arrived);
+                    else if (kmax == 1) acc = tile_dot<1, true>(gt, want, col, val, add, 1, 1, stalled, arrived);
+                    else acc = tile_dot<4, true>(gt, want, col, val, add, 4, 4, stalled, arrived);
+                } else acc = tile_dot<N, false>(gt, want, col, val, add, kmax, cnt, stalled, arrived);
                 if (kmax == 0) acc = arrived();
                 if (stalled) break;
                 if (lng) {
@@ -308,7 +314,7 @@ __global__ void __launch_bounds__(NT, 1) k_block(const __grid_constant__ BlockPl
             const int2 d = *reinterpret_cast<const int2 *>(blk_smem + tile);
             const int r = d.x + lane, src = it & 1;
             const unsigned tag = seq + (unsigned)it + 1;
-            double *z = reinterpret_cast<double *>(blk_smem + tile + sizeof(BlockTile)) + lane;
+            double *z = reinterpret_cast<double *>(blk_smem + tile + kTileHead) + lane;
             const BlockLp &L = lps[ONE ? 0 : tile_lp(d.y)];
             const bool keep = it == (ONE ? nit : L.lim) - 1;
             if (lane >= tile_rows(d.y)) continue;

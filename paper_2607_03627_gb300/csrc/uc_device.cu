@@ -2494,24 +2494,19 @@ static void build_tables(const uc_session &X, const std::vector<char> &mask, std
     sa.insert(sa.end(), sd.begin(), sd.end());
 }
 
-// Largest lg in 5, 4, 3 such that entry q of row s of every group of 2^lg of the
-// rows [a, b) of M (the last may be short) is (col_q + s, val_q), values as stored;
-// 0 if there is none.  v32: the FP32 values, if M is stored so.
-static int tile_group(const Csr &M, const std::vector<float> &v32, int a, int b) {
-    int lg = 5;
+// bit r - a: row r of M, of rows [a, b), does not go on a run of the rows before it
+// (see BlockTile); values as stored, v32: the FP32 values, if M is stored so
+static unsigned tile_runs(const Csr &M, const std::vector<float> &v32, int a, int b) {
+    unsigned runs = 1;
     for (int r = a + 1; r < b; r++) {
-        while (lg >= 3) {
-            const int s = (r - a) & ((1 << lg) - 1), e0 = M.rowptr[r - s], e = M.rowptr[r], k = M.rowptr[r + 1] - e;
-            bool same = M.rowptr[r - s + 1] - e0 == k;
-            for (int q = 0; s > 0 && same && q < k; q++)
-                same = M.colidx[e + q] == M.colidx[e0 + q] + s &&
-                       (v32.empty() ? M.val[e + q] == M.val[e0 + q] : v32[e + q] == v32[e0 + q]);
-            if (same) break;
-            lg--;
-        }
-        if (lg < 3) return 0;
+        const int p = M.rowptr[r - 1], e = M.rowptr[r], k = M.rowptr[r + 1] - e;
+        bool same = e - p == k;
+        for (int q = 0; same && q < k; q++)
+            same = M.colidx[e + q] == M.colidx[p + q] + 1 &&
+                   (v32.empty() ? M.val[e + q] == M.val[p + q] : v32[e + q] == v32[p + q]);
+        if (!same) runs |= 1u << (r - a);
     }
-    return lg;
+    return runs;
 }
 
 // Tiles of the resident block kernel for the LPs in `mask`, dealt to the warps of
@@ -2526,6 +2521,10 @@ static void plan_block(uc_session &X, const std::vector<char> &mask, std::vector
     X.block = false;
     if (!X.block_able) return;
     std::vector<BlockTile> t[2];   // dual, primal
+    auto bytes_of = [](const BlockTile &T) {
+        const int runs = __builtin_popcount(T.runs);
+        return tile_bytes(tile_stride(T.kmax, runs), runs);
+    };
     int64_t bytes = 0;
     for (int i = 0; i < X.k; i++) {
         if (!mask[i]) continue;
@@ -2539,17 +2538,17 @@ static void plan_block(uc_session &X, const std::vector<char> &mask, std::vector
                     kmax = std::max(kmax, M.rowptr[r + 1] - M.rowptr[r]);
                     kmin = std::min(kmin, M.rowptr[r + 1] - M.rowptr[r]);
                 }
-                const int lg = tile_group(M, primal ? v.AT_val32 : v.A_val32, s, e);
-                const int kind = lg && kmin == kmax && kmax >= 1 && kmax <= kUniform ? TILE_UNIFORM : TILE_ANY;
-                t[primal].push_back(BlockTile{(int)(base + s), tile_info(e - s, kind, lg, primal, ineq, i), kmax, 0});
-                bytes += tile_bytes(kmax, lg);
+                const unsigned runs = tile_runs(M, primal ? v.AT_val32 : v.A_val32, s, e);
+                const int kind = kmin == kmax && kmax >= 1 && kmax <= kUniform ? TILE_UNIFORM : TILE_ANY;
+                t[primal].push_back(BlockTile{(int)(base + s), tile_info(e - s, kind, primal, ineq, i), kmax, runs, 0, {}});
+                bytes += bytes_of(t[primal].back());
             }
         };
         cut(v.AT, 0, n - nl, X.coff[i], true, false);
         for (int j = n - nl; j < n; j++) {
             const int kmax = (v.AT.rowptr[j + 1] - v.AT.rowptr[j] + 31) / 32;
-            t[1].push_back(BlockTile{(int)(X.coff[i] + j), tile_info(1, TILE_LONG, 0, true, false, i), kmax, 0});
-            bytes += tile_bytes(kmax, 0);
+            t[1].push_back(BlockTile{(int)(X.coff[i] + j), tile_info(1, TILE_LONG, true, false, i), kmax, ~0u, 0, {}});
+            bytes += bytes_of(t[1].back());
         }
         cut(v.A, 0, m_eq, X.roff[i], false, false);
         cut(v.A, m_eq, m, X.roff[i], false, true);
@@ -2564,8 +2563,8 @@ static void plan_block(uc_session &X, const std::vector<char> &mask, std::vector
     std::vector<std::vector<const BlockTile *>> mine[2];
     for (int ph = 0; ph < 2; ph++) {
         mine[ph].resize(S);
-        std::stable_sort(t[ph].begin(), t[ph].end(), [](const BlockTile &a, const BlockTile &b) {
-            return a.kmax != b.kmax ? a.kmax > b.kmax : tile_lg(a.info) < tile_lg(b.info);
+        std::stable_sort(t[ph].begin(), t[ph].end(), [&](const BlockTile &a, const BlockTile &b) {
+            return a.kmax != b.kmax ? a.kmax > b.kmax : bytes_of(a) > bytes_of(b);
         });
         for (int64_t i = 0; i < (int64_t)t[ph].size(); i++) mine[ph][ph ? i % S : S - 1 - i % S].push_back(&t[ph][i]);
     }
@@ -2584,7 +2583,7 @@ static void plan_block(uc_session &X, const std::vector<char> &mask, std::vector
             const BlockWarp &wp = warps[(size_t)c * W + w];
             for (int q = wp.first; q < wp.first + wp.count; q++) {
                 tiles[q].smem = (int)at;
-                at += tile_bytes(tiles[q].kmax, tile_lg(tiles[q].info));
+                at += bytes_of(tiles[q]);
             }
         }
         most = std::max(most, at);

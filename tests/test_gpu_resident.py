@@ -50,8 +50,8 @@ def test_resident_kernel_equals_row_kernels(B, buses, periods, units, value_bits
     _same(B, a, B.uc_solve(ps, tol=0.0, max_iter=100, n_eval=2, use_graph=False)[0], ps)
 
 
-# shared entries in groups of 8, 16 and 32 rows, in none (periods of 10 and 31), and the
-# largest CTAs (2,000 buses of 48 periods: more than five tiles per warp)
+# runs of rows with shared entries that begin on tile and group edges (8, 16, 32 periods)
+# and off them (10, 31), and the largest CTAs (2,000 buses of 48 periods: more than five tiles per warp)
 @pytest.mark.parametrize("buses,periods,units", [(70, 8, 9), (60, 10, 9), (50, 16, 6), (45, 32, 6), (64, 31, 8), (2000, 48, 240)])
 @pytest.mark.parametrize("value_bits", [64, 32])
 def test_resident_kernel_with_shared_entries(B, buses, periods, units, value_bits):
