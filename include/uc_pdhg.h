@@ -170,9 +170,11 @@ typedef struct {
     int stages;                  /* staged kernels: chunks in flight per CTA, 2..8 (0: default 2);
                                     results do not depend on it (tuning knob) */
     int lanes;                   /* 1: the session's 2 or 4 LPs share one scaled matrix (e.g. requests
-                                    on one grid presolved with uc_presolve_reuse); it is stored once
-                                    and the LPs' vectors are interleaved, so every row is read once
-                                    for all of them (Halpern, row kernels; UC_EINVAL otherwise).
+                                    on one grid presolved with uc_presolve_reuse); LPs that fit into
+                                    the SMs' shared memory run there one beside another; otherwise the
+                                    matrix is stored once and the LPs' vectors are interleaved, so every
+                                    row is read once for all of them (Halpern, row kernels; UC_EINVAL
+                                    otherwise; spmv_kernel 1: always interleaved).
                                     Iterates are those of separate solves, bit for bit. */
     int adaptive_step;           /* 1: PDLP's adaptive step size (Applegate et al. 2021, Sec. 3.1) for
                                     algorithm 1: each iteration is an attempt with a trial step eta,
@@ -312,7 +314,7 @@ int uc_presolved_strided_groups(const uc_presolved *ps, int transpose, int64_t *
 int uc_solve(const uc_presolved *ps, const uc_solve_opts *opts, void *stream, uc_result **out);
 
 /* Solve k presolved LPs at once: their matrices are packed block-diagonally
- * (or, with opts->lanes, stored once for 2 or 4 LPs that share it) and every
+ * (or, with opts->lanes, may be stored once for 2 or 4 LPs that share it) and every
  * iteration launches one primal and one dual kernel for all of them; each LP
  * keeps its own step sizes, restarts and stopping test and freezes when it
  * converges.  outs[i] receives LP i's result.  Returns UC_OK if every LP
@@ -321,8 +323,8 @@ int uc_solve_batch(const uc_presolved *const *ps, int k, const uc_solve_opts *op
                    uc_result **outs);
 
 /* Device-resident sessions.  A session uploads k presolved LPs once (matrices
- * block-diagonal, or one shared matrix with interleaved vectors when
- * opts->lanes is set; per-LP vectors, start points, CUDA graph of n_eval
+ * block-diagonal, or one shared matrix with interleaved vectors where
+ * opts->lanes asks for it; per-LP vectors, start points, CUDA graph of n_eval
  * iterations) and then solves them any number of times; it is what uc_solve
  * and uc_solve_batch use internally, and what a server uses to keep
  * instances resident, warm-start re-solves and refill finished slots while

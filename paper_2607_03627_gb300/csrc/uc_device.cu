@@ -1754,7 +1754,8 @@ struct uc_session {
     std::vector<char> tabled;     // LPs whose CTAs are in the current tables and graph
     int cap_sp = 0, cap_sd = 0, cap_se = 0, cap_sa = 0;
     // shared-matrix ("lanes") sessions: K LPs with one scaled matrix, stored
-    // once, vectors interleaved (element j of LP r at j*K + r); K = 1 otherwise
+    // once, vectors interleaved (element j of LP r at j*K + r); K = 1 otherwise,
+    // also where the resident kernel takes the LPs one after another
     int K = 1;
     int64_t Mr = 0, Nr = 0;       // rows of A and of A^T as stored
     // primal feasibility polishing in progress: LPs reset now stop on this
@@ -2703,8 +2704,9 @@ static int retable(uc_session &X, const std::vector<char> &mask) {
 
 static bool live_status(int st) { return st == RUNNING || st == NEEDS_INIT; }
 
-static int session_create(const PsData *const *Pp, const std::shared_ptr<const PsData> *owners, int k,
-                          const uc_solve_opts &o, cudaStream_t user_stream, uc_session **out) {
+// split: a lanes session may store its LPs one after another (see below)
+static int session_create_as(const PsData *const *Pp, const std::shared_ptr<const PsData> *owners, int k,
+                             const uc_solve_opts &o, cudaStream_t user_stream, bool split, uc_session **out) {
     *out = nullptr;
     if (k < 1) { set_error("need at least one LP"); return UC_EINVAL; }
     if (o.n_eval < 2 || (o.n_eval & 1)) { set_error("n_eval must be even and >= 2"); return UC_EINVAL; }
@@ -2774,27 +2776,31 @@ static int session_create(const PsData *const *Pp, const std::shared_ptr<const P
                 set_error("lanes sessions need LPs with one scaled matrix (LP %d differs from LP 0)", i);
                 return UC_EINVAL;
             }
-        X->K = k;
-        X->cta = 128;   // the lanes kernels are built for 128-thread CTAs
     }
-    X->roff.assign(k + 1, 0); X->coff.assign(k + 1, 0); X->zoff.assign(k + 1, 0);
-    if (X->K > 1) {
-        // one structure: every LP starts at row, column and entry 0
-        X->M = (int64_t)Pp[0]->m() * X->K; X->N = (int64_t)Pp[0]->n() * X->K; X->Z = Pp[0]->A.nnz();
-        X->Mr = Pp[0]->m(); X->Nr = Pp[0]->n();
-        X->roff[k] = X->Mr; X->coff[k] = X->Nr; X->zoff[k] = X->Z;
-    } else {
-        for (int i = 0; i < k; i++) {
-            X->roff[i + 1] = X->roff[i] + Pp[i]->m();
-            X->coff[i + 1] = X->coff[i] + Pp[i]->n();
-            X->zoff[i + 1] = X->zoff[i] + Pp[i]->A.nnz();
+    // offsets of the LPs; interleaved: one structure, every LP starts at row, column and entry 0
+    auto lay_out = [&](bool interleaved) {
+        X->K = interleaved ? k : 1;
+        X->roff.assign(k + 1, 0); X->coff.assign(k + 1, 0); X->zoff.assign(k + 1, 0);
+        if (interleaved) {
+            X->M = (int64_t)Pp[0]->m() * k; X->N = (int64_t)Pp[0]->n() * k; X->Z = Pp[0]->A.nnz();
+            X->Mr = Pp[0]->m(); X->Nr = Pp[0]->n();
+            X->roff[k] = X->Mr; X->coff[k] = X->Nr; X->zoff[k] = X->Z;
+        } else {
+            for (int i = 0; i < k; i++) {
+                X->roff[i + 1] = X->roff[i] + Pp[i]->m();
+                X->coff[i + 1] = X->coff[i] + Pp[i]->n();
+                X->zoff[i + 1] = X->zoff[i] + Pp[i]->A.nnz();
+            }
+            X->M = X->roff[k]; X->N = X->coff[k]; X->Z = X->zoff[k];
+            X->Mr = X->M; X->Nr = X->N;
         }
-        X->M = X->roff[k]; X->N = X->coff[k]; X->Z = X->zoff[k];
-        X->Mr = X->M; X->Nr = X->N;
+        // row indices are also stored shifted left by one bit in the evaluation table
+        return X->M < (1LL << 30) && X->N < INT32_MAX && X->Z < INT32_MAX;
+    };
+    if (!lay_out(o.lanes && !split)) {
+        split = false;
+        if (!o.lanes || !lay_out(true)) { set_error("batch too large for int32 indices"); return UC_EINVAL; }
     }
-    const int64_t M = X->M, N = X->N, Z = X->Z;
-    // row indices are also stored shifted left by one bit in the evaluation table
-    if (M >= (1LL << 30) || N >= INT32_MAX || Z >= INT32_MAX) { set_error("batch too large for int32 indices"); return UC_EINVAL; }
 
     X->rpt.assign(k, 1);
     X->m_eq.assign(k, 0);
@@ -2821,6 +2827,34 @@ static int session_create(const PsData *const *Pp, const std::shared_ptr<const P
         int rc = staged_setup(*X);
         if (rc) return rc;
     }
+    // resident block kernel: Halpern row sessions
+    std::vector<BlockTile> tiles;
+    std::vector<BlockWarp> warps;
+    {
+        int dev = 0, coop = 0;
+        UC_CUDA(cudaGetDevice(&dev));
+        UC_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
+        UC_CUDA(cudaDeviceGetAttribute(&X->sms, cudaDevAttrMultiProcessorCount, dev));
+        UC_CUDA(cudaDeviceGetAttribute(&X->blk_smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+        X->blk_smem_max -= 1024;   // the kernel's static part
+        X->block_able = coop && o.spmv_kernel == 0 && X->algo == ALG_HALPERN && X->K == 1 && k <= kBlockMaxLps &&
+                        o.n_eval <= kBlockMaxEval;
+        if (X->block_able)
+            for (int nt : {kSmallThreads, kMidThreads, kBigThreads})
+                UC_CUDA(cudaFuncSetAttribute(block_kernel(*X, nt), cudaFuncAttributeMaxDynamicSharedMemorySize, X->blk_smem_max));
+        plan_block(*X, std::vector<char>(k, 1), tiles, warps);
+        if (k == 1 && !X->block) X->block_able = false;   // no subset of its LPs fits either
+    }
+    // A lanes session whose LPs fit into shared memory one after another runs the
+    // resident kernel: two LPs of 474 k rows and columns 14.3 us per iteration (the
+    // interleaved kernels 18.0), four of 95 k 6.9 (13.0).  Its tables hold all LPs to its
+    // end, and the matrix is stored once per LP.  Else the vectors are interleaved.
+    if (o.lanes && !X->block) {
+        lay_out(true);
+        X->block_able = false;
+        X->cta = 128;   // the lanes kernels are built for 128-thread CTAs
+    }
+    const int64_t M = X->M, N = X->N, Z = X->Z;
     // CTA tables for every LP (their sizes are the capacities of the device tables)
     std::vector<Seg> sp, sd, se, sa;
     std::vector<InstRange> ranges;
@@ -2839,24 +2873,6 @@ static int session_create(const PsData *const *Pp, const std::shared_ptr<const P
     X->n_sp = X->cap_sp = (int)sp.size(); X->n_sd = X->cap_sd = (int)sd.size();
     X->n_se = X->cap_se = (int)se.size(); X->n_sa = X->cap_sa = (int)sa.size();
 
-    // resident block kernel: Halpern row sessions
-    std::vector<BlockTile> tiles;
-    std::vector<BlockWarp> warps;
-    {
-        int dev = 0, coop = 0;
-        UC_CUDA(cudaGetDevice(&dev));
-        UC_CUDA(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
-        UC_CUDA(cudaDeviceGetAttribute(&X->sms, cudaDevAttrMultiProcessorCount, dev));
-        UC_CUDA(cudaDeviceGetAttribute(&X->blk_smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-        X->blk_smem_max -= 1024;   // the kernel's static part
-        X->block_able = coop && o.spmv_kernel == 0 && X->algo == ALG_HALPERN && X->K == 1 && k <= kBlockMaxLps &&
-                        o.n_eval <= kBlockMaxEval;
-        if (X->block_able)
-            for (int nt : {kSmallThreads, kMidThreads, kBigThreads})
-                UC_CUDA(cudaFuncSetAttribute(block_kernel(*X, nt), cudaFuncAttributeMaxDynamicSharedMemorySize, X->blk_smem_max));
-        plan_block(*X, all, tiles, warps);
-        if (k == 1 && !X->block) X->block_able = false;   // no subset of its LPs fits either
-    }
     Layout &L = X->L;
     size_t off = 0;
     // 16 bytes of slack after every array: the staged kernels' copies round
@@ -3179,7 +3195,7 @@ static int session_run(uc_session &X, int max_replays) {
                 live += want[i];
                 tab += X.tabled[i];
             }
-            if (X.K == 1 && live > 0 && 4 * live <= 3 * tab) {   // lanes sessions keep one table
+            if (!X.o.lanes && live > 0 && 4 * live <= 3 * tab) {   // lanes sessions keep one table
                 // drain the replay still in flight, then rebuild for the live LPs only
                 UC_CUDA(cudaStreamSynchronize(s));
                 checked = launched;
@@ -3324,6 +3340,14 @@ static int session_result(uc_session &X, int i, uc_result **out) {
     X.active[i] = 0;
     *out = guard.release();
     return status;
+}
+
+static int session_create(const PsData *const *Pp, const std::shared_ptr<const PsData> *owners, int k,
+                          const uc_solve_opts &o, cudaStream_t user_stream, uc_session **out) {
+    int rc = session_create_as(Pp, owners, k, o, user_stream, true, out);
+    // the interleaved layout holds the matrix once
+    if (rc == UC_ENOMEM && o.lanes) rc = session_create_as(Pp, owners, k, o, user_stream, false, out);
+    return rc;
 }
 
 static int session_update_lp(uc_session &X, int i, const std::shared_ptr<const PsData> &np) {

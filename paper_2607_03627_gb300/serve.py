@@ -14,9 +14,10 @@ base LP's scaling is reused) runs on a thread pool as requests arrive.
 
 Because every slot's arithmetic is independent and deterministic, a request
 returns the same iterates and solution alone or in the mix (tested).  With 2
-or 4 slots the session is a shared-matrix ("lanes") session: the base matrix
-is stored once, the slots' vectors are interleaved, and every matrix row is
-read once for all slots.
+or 4 slots the session is a shared-matrix ("lanes") session: slots that fit
+into the SMs' shared memory run there one beside another; otherwise the base
+matrix is stored once, the slots' vectors are interleaved, and every matrix row
+is read once for all slots.
 """
 from __future__ import annotations
 
@@ -80,8 +81,7 @@ class Server:
         fit = max(1, int(hbm_budget_gb * 1e9 // per_slot))
         self.slots = max(1, min(slots, fit))
         self.bytes_per_slot = per_slot
-        # 2 or 4 slots share one stored matrix and interleave their vectors
-        # (a lanes session) unless told otherwise
+        # 2 or 4 slots are a shared-matrix (lanes) session unless told otherwise
         self.lanes = (self.slots in (2, 4)) if lanes is None else (bool(lanes) and self.slots in (2, 4))
         self.sess = B.Session([self.base_ps] * self.slots, tol=tol, max_iter=max_iter, lanes=self.lanes)
         self.pool = cf.ThreadPoolExecutor(max_workers=presolve_workers)

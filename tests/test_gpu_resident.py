@@ -86,6 +86,32 @@ def test_resident_batch_rebuilt_as_it_shrinks(B):
         _same(B, B.uc_solve(ps, tol=1e-4, max_iter=20_000)[0], outs[0][i], ps)
 
 
+@pytest.mark.parametrize("slots", [2, 4])
+@pytest.mark.parametrize("value_bits", [64, 32])
+def test_shared_matrix_session_resident_equals_interleaved(B, slots, value_bits):
+    # LPs of one grid: in shared memory one beside another, or interleaved (spmv_kernel 1)
+    base = _grid(5, 60, 24, 8)
+    ps0 = B.uc_presolve(B.uc_build_lp(base), value_bits=value_bits, power_max_iter=20)
+    pss = [B.uc_presolve_reuse(ps0, B.uc_build_lp(ucgen.served_request(base, 5, r))) for r in range(slots + 1)]
+    for n_eval, budget in ((64, 1), (64, 130), (2, 64)):
+        kw = dict(tol=0.0, max_iter=budget, n_eval=n_eval, lanes=True)
+        for ps, ra, rb in zip(pss, B.uc_solve_batch(pss[:slots], spmv_kernel=1, **kw)[0], B.uc_solve_batch(pss[:slots], **kw)[0]):
+            _same(B, ra, rb, ps)
+    outs = []
+    for kernel in (1, 0):                # to the end at different times, then one slot refilled alone
+        s = B.Session(pss[:slots], tol=1e-3, max_iter=20_000, lanes=True, spmv_kernel=kernel)
+        s.reset(-1)
+        s.run()
+        outs.append([s.result(i)[0] for i in range(slots)])
+        s.update_lp(1, pss[slots])
+        s.reset(1)
+        s.run()
+        outs[-1].append(s.result(1)[0])
+        s.close()
+    for i, (ra, rb) in enumerate(zip(*outs)):
+        _same(B, ra, rb, pss[i])
+
+
 def test_resident_sessions_on_several_streams(B):
     import concurrent.futures as cf
 
