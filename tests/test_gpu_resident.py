@@ -112,6 +112,32 @@ def test_shared_matrix_session_resident_equals_interleaved(B, slots, value_bits)
         _same(B, ra, rb, pss[i])
 
 
+# one host thread and several, the slots' largest LP and a smaller one
+@pytest.mark.parametrize("buses", [(40, 20), (500, 30)])
+@pytest.mark.parametrize("reorder", [True, False])
+def test_slot_takes_another_lp(B, buses, reorder):
+    grids = [_grid(s, b, 24, 4) for s, b in enumerate(buses)]
+    firsts = [B.uc_presolve(B.uc_build_lp(P), power_max_iter=20) for P in grids]
+    s = B.Session(firsts, tol=0.0, max_iter=130, reorder=reorder)
+    s.reset(-1)
+    s.run()
+    for slot in (0, 1):
+        other = B.uc_presolve_reuse(firsts[slot], B.uc_build_lp(ucgen.served_request(grids[slot], slot, 3)))
+        with pytest.raises(B.UCError):
+            s.update_lp(1 - slot, other)
+        s.update_lp(slot, other)
+        s.reset(slot)
+        s.run()
+        got = s.result(slot)[0]
+        _same(B, B.uc_solve(other, tol=0.0, max_iter=130, reorder=reorder)[0], got, other)
+        _, yw = B.uc_get_iterate(got, 2, *B.uc_presolved_dims(other)[:2])
+        s.set_start(slot, None, yw, 0.5)     # a start of the new LP's
+        s.reset(slot)
+        s.run()
+        _same(B, B.uc_solve(other, tol=0.0, max_iter=130, reorder=reorder, warm_y=yw, warm_omega=0.5)[0], s.result(slot)[0], other)
+    s.close()
+
+
 def test_resident_sessions_on_several_streams(B):
     import concurrent.futures as cf
 
