@@ -3744,67 +3744,96 @@ __global__ void __launch_bounds__(kThreads, kNoAllocCtas) k_kkt_noalloc(uc_devic
 // ---------------------------------------------------------------------------
 // ||A||_2 for presolve on the device: power iteration on A^T A
 // ---------------------------------------------------------------------------
-// State: st[0] = lambda, st[1] = previous lambda; *done: 0 running, 1 converged,
-// 2 lambda == 0.  Every kernel returns at once when *done is set, so a fixed
-// number of launches can be queued and the host only polls.
-constexpr int kPwThreads = 128;
+// A step is two launches: t = scale A w, then w = A^T t with |w| and the stopping
+// test by the CTA that ends last.  The iterate is kept in the range by a power of two
+// instead of divided by its norm: exact, so v = scale w loses nothing, and lambda =
+// |A^T A v| / |v| with |v| = scale |w|.  Every kernel returns at once when done is set,
+// so a fixed number of launches can be queued and the host only polls.
+//
+// Four entries' loads at a time; the first four and the row pointers come before the
+// wait for the kernel before (programmatic dependent launch).  3,000 buses of 48
+// periods (948 k rows and columns, 1.3 M entries): 33 us per step; as two products
+// of one entry at a time, a norm by one CTA and a pass of divisions 46.  Small LPs 9 us
+// (launches), large ones are bound by the gathers, which the presolved order spreads
+// over L2: neither more threads per SM (64 warps 33.6) nor smaller CTAs (33.0) matter.
+struct PwState {
+    double lambda, prev, scale, vnorm;   // last estimates; of the current iterate
+    int done;                            // 0 running, 1 converged, 2 lambda == 0
+    unsigned ended;                      // CTAs of the norm that ended (wraps to zero)
+};
+constexpr int kPwThreads = 256;
 
-// y = M x, one thread per row; with part, CTA b also writes sum of y_i^2 over
-// its rows (warp shuffles, then warps in order: a fixed order).
-__global__ void __launch_bounds__(kPwThreads) k_pw_spmv(const int32_t *__restrict__ rp, const int32_t *__restrict__ ci,
-                                                        const double *__restrict__ val, int rows,
-                                                        const double *__restrict__ x, double *__restrict__ y,
-                                                        double *__restrict__ part, const int *__restrict__ done) {
-    if (*done) return;
-    const int i = blockIdx.x * kPwThreads + threadIdx.x;
-    double s = 0.0;
-    if (i < rows) {
-        for (int k = rp[i]; k < rp[i + 1]; k++) s += val[k] * x[ci[k]];
-        y[i] = s;
-    }
-    if (!part) return;
-    double sq = s * s;
+// sum over the CTA, valid in thread 0: warp shuffles, then the warps in order
+__device__ __forceinline__ double pw_block_sum(double v, double *sh) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) sq += __shfl_down_sync(0xffffffffu, sq, o);
-    __shared__ double sh[kPwThreads / 32];
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = sq;
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = sh[0];
+    double t = sh[0];
+    if (threadIdx.x == 0)
         for (int w = 1; w < kPwThreads / 32; w++) t += sh[w];
-        part[blockIdx.x] = t;
-    }
+    return t;
 }
 
-// lambda = sqrt(sum of the CTA partials), one CTA of 1024 threads (strided
-// partial sums, then a tree: a fixed order); the stopping test of the step.
-__global__ void __launch_bounds__(1024) k_pw_norm(const double *__restrict__ part, int np, double *st, int *done,
-                                                  double tol) {
-    if (*done) return;
-    __shared__ double sh[1024];
-    double s = 0.0;
-    for (int p = threadIdx.x; p < np; p += 1024) s += part[p];
-    sh[threadIdx.x] = s;
-    __syncthreads();
-    for (int h = 512; h > 0; h >>= 1) {
-        if (threadIdx.x < h) sh[threadIdx.x] += sh[threadIdx.x + h];
-        __syncthreads();
+// one thread per row; NORM: y = M x and the step's norm, else y = scale M x
+template <bool NORM>
+__global__ void __launch_bounds__(kPwThreads) k_pw_spmv(const int32_t *__restrict__ rp, const int32_t *__restrict__ ci,
+                                                        const double *__restrict__ val, int rows, const double *x, double *y,
+                                                        double *part, PwState *st, double tol) {
+    const int i = blockIdx.x * kPwThreads + threadIdx.x;
+    int k0 = 0, k1 = 0, c[4];
+    double a[4], s = 0.0;
+    if (i < rows) { k0 = rp[i]; k1 = rp[i + 1]; }
+#pragma unroll
+    for (int q = 0; q < 4; q++) if (k0 + q < k1) { c[q] = ld_stream(ci + k0 + q); a[q] = ld_stream(val + k0 + q); }
+    pdl_wait();
+    pdl_trigger();
+    if (__ldcg(&st->done)) return;
+#pragma unroll 1
+    while (__any_sync(0xffffffffu, k0 < k1)) {
+        double g[4];
+#pragma unroll
+        for (int q = 0; q < 4; q++) if (k0 + q < k1) g[q] = x[c[q]];
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            if (!__any_sync(0xffffffffu, k0 + q < k1)) break;
+            if (k0 + q < k1) s = fma(a[q], g[q], s);
+        }
+        k0 += 4;
+#pragma unroll
+        for (int q = 0; q < 4; q++) if (k0 + q < k1) { c[q] = ld_stream(ci + k0 + q); a[q] = ld_stream(val + k0 + q); }
     }
+    if (!NORM) {
+        if (i < rows) y[i] = s * __ldcg(&st->scale);
+        return;
+    }
+    if (i < rows) y[i] = s;
+    __shared__ double sh[kPwThreads / 32];
+    __shared__ bool last;
+    const double mine = pw_block_sum(s * s, sh);
     if (threadIdx.x == 0) {
-        const double lam = sqrt(sh[0]);
-        st[0] = lam;
-        if (lam == 0.0) *done = 2;
-        else if (fabs(lam - st[1]) <= tol * lam) *done = 1;
-        else st[1] = lam;
+        __stcg(part + blockIdx.x, mine);
+        __threadfence();
+        last = atomicInc(&st->ended, gridDim.x - 1) == gridDim.x - 1;
     }
-}
-
-// v = w / lambda (skipped once the iteration has stopped: v is not used again)
-__global__ void k_pw_div(const double *__restrict__ w, double *__restrict__ v, int n, const double *st,
-                         const int *done) {
-    if (*done) return;
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j < n) v[j] = w[j] / st[0];
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    double t[4] = {};
+    for (int p = threadIdx.x; p < (int)gridDim.x; p += 4 * kPwThreads)
+#pragma unroll
+        for (int q = 0; q < 4; q++)
+            if (p + q * kPwThreads < (int)gridDim.x) t[q] += __ldcg(part + p + q * kPwThreads);
+    const double sum = pw_block_sum((t[0] + t[1]) + (t[2] + t[3]), sh);
+    if (threadIdx.x != 0) return;
+    const double nrm = sqrt(sum), lam = nrm / st->vnorm;
+    st->lambda = lam;
+    if (lam == 0.0) st->done = 2;
+    else if (fabs(lam - st->prev) <= tol * lam) st->done = 1;
+    else st->prev = lam;
+    const int e = max(-1000, min(1000, ((__double2hiint(nrm) >> 20) & 0x7ff) - 1023));
+    st->scale = __hiloint2double((1023 - e) << 20, 0);
+    st->vnorm = nrm * st->scale;
 }
 
 }  // namespace dev
@@ -3827,8 +3856,8 @@ int device_power_norm(const Csr &A, const Csr &AT, int max_iter, double tol, dou
     const size_t o_arp = take(sizeof(int32_t) * (m + 1)), o_aci = take(sizeof(int32_t) * nnz),
                  o_av = take(sizeof(double) * nnz), o_trp = take(sizeof(int32_t) * (n + 1)),
                  o_tci = take(sizeof(int32_t) * nnz), o_tv = take(sizeof(double) * nnz),
-                 o_v = take(sizeof(double) * n), o_t = take(sizeof(double) * m), o_w = take(sizeof(double) * n),
-                 o_part = take(sizeof(double) * np), o_st = take(sizeof(double) * 2), o_done = take(sizeof(int));
+                 o_t = take(sizeof(double) * m), o_w = take(sizeof(double) * n), o_part = take(sizeof(double) * np),
+                 o_st = take(sizeof(PwState));
     cudaStream_t s = nullptr;
     UC_CUDA(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
     char *D = nullptr;
@@ -3843,13 +3872,12 @@ int device_power_norm(const Csr &A, const Csr &AT, int max_iter, double tol, dou
     if (rc == UC_OK && (e = cudaMallocHost((void **)&h_done, sizeof(int))) != cudaSuccess) fail(e, "cudaMallocHost");
     if (rc == UC_OK) {
         std::vector<double> v0((size_t)n, 1.0 / std::sqrt((double)n));
-        const double st0[2] = {0.0, 0.0};
-        const int zero = 0;
+        const PwState st0{0.0, 0.0, 1.0, 1.0, 0, 0};
         struct Up { size_t o; const void *src; size_t bytes; } ups[] = {
             {o_arp, A.rowptr.data(), sizeof(int32_t) * (m + 1)}, {o_aci, A.colidx.data(), sizeof(int32_t) * nnz},
             {o_av, A.val.data(), sizeof(double) * nnz}, {o_trp, AT.rowptr.data(), sizeof(int32_t) * (n + 1)},
             {o_tci, AT.colidx.data(), sizeof(int32_t) * nnz}, {o_tv, AT.val.data(), sizeof(double) * nnz},
-            {o_v, v0.data(), sizeof(double) * n}, {o_st, st0, sizeof(st0)}, {o_done, &zero, sizeof(int)}};
+            {o_w, v0.data(), sizeof(double) * n}, {o_st, &st0, sizeof(st0)}};
         for (const Up &u : ups)
             if (rc == UC_OK && (e = cudaMemcpyAsync(D + u.o, u.src, u.bytes, cudaMemcpyHostToDevice, s)) != cudaSuccess)
                 fail(e, "cudaMemcpyAsync");
@@ -3860,22 +3888,21 @@ int device_power_norm(const Csr &A, const Csr &AT, int max_iter, double tol, dou
         const int32_t *arp = (const int32_t *)(D + o_arp), *aci = (const int32_t *)(D + o_aci);
         const int32_t *trp = (const int32_t *)(D + o_trp), *tci = (const int32_t *)(D + o_tci);
         const double *av = (const double *)(D + o_av), *tv = (const double *)(D + o_tv);
-        double *v = (double *)(D + o_v), *t = (double *)(D + o_t), *w = (double *)(D + o_w);
-        double *part = (double *)(D + o_part), *st = (double *)(D + o_st);
-        int *done = (int *)(D + o_done);
+        double *t = (double *)(D + o_t), *w = (double *)(D + o_w), *part = (double *)(D + o_part);
+        PwState *st = (PwState *)(D + o_st);
         const int gm = (m + kPwThreads - 1) / kPwThreads, gn = np;
         constexpr int kPoll = 64;   // steps queued between polls of the stop flag
         for (int it = 0; it < max_iter && rc == UC_OK;) {
             const int batch = std::min(kPoll, max_iter - it);
-            for (int b = 0; b < batch; b++) {
-                k_pw_spmv<<<gm, kPwThreads, 0, s>>>(arp, aci, av, m, v, t, nullptr, done);
-                k_pw_spmv<<<gn, kPwThreads, 0, s>>>(trp, tci, tv, n, t, w, part, done);
-                k_pw_norm<<<1, 1024, 0, s>>>(part, np, st, done, tol);
-                k_pw_div<<<gn, kPwThreads, 0, s>>>(w, v, n, st, done);
+            for (int b = 0; b < batch && e == cudaSuccess; b++) {
+                e = launch_k(k_pw_spmv<false>, gm, kPwThreads, s, true, arp, aci, av, m, (const double *)w, t, (double *)nullptr, st, tol);
+                if (e == cudaSuccess)
+                    e = launch_k(k_pw_spmv<true>, gn, kPwThreads, s, true, trp, tci, tv, n, (const double *)t, w, part, st, tol);
             }
+            if (e != cudaSuccess) { fail(e, "kernel launch"); break; }
             it += batch;
             if ((e = cudaGetLastError()) != cudaSuccess) { fail(e, "kernel launch"); break; }
-            if ((e = cudaMemcpyAsync(h_done, done, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
+            if ((e = cudaMemcpyAsync(h_done, &st->done, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
                 (e = cudaStreamSynchronize(s)) != cudaSuccess) {
                 fail(e, "power iteration");
                 break;
@@ -3884,7 +3911,7 @@ int device_power_norm(const Csr &A, const Csr &AT, int max_iter, double tol, dou
         }
         // every pass of the loop ends with a synchronisation, so *h_done is current
         double lam = 0.0;
-        if (rc == UC_OK && ((e = cudaMemcpyAsync(&lam, st, sizeof(double), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
+        if (rc == UC_OK && ((e = cudaMemcpyAsync(&lam, &st->lambda, sizeof(double), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
                             (e = cudaStreamSynchronize(s)) != cudaSuccess))
             fail(e, "result download");
         if (rc == UC_OK) *out = (*h_done == 2) ? 0.0 : std::sqrt(lam);
