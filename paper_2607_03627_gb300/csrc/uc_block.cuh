@@ -62,9 +62,9 @@ struct __align__(16) BlockTile {
     unsigned info;   // see tile_info
     int kmax;
     unsigned runs;
-    int smem, pad[3];
+    int smem, img, pad[2];   // where it is: byte in shared memory, 16-byte unit of the image
 };
-constexpr int kTileHead = 16;
+constexpr int kTileHead = 16, kTileOwn = kTileHead + kTileRows * 8;   // before the entries
 __host__ __device__ constexpr unsigned tile_info(int rows, int kind, bool primal, bool ineq, int lp) {
     return (unsigned)rows | (unsigned)kind << 6 | (unsigned)primal << 8 | (unsigned)ineq << 9 | (unsigned)lp << 10;
 }
@@ -76,7 +76,7 @@ __host__ __device__ constexpr int tile_lp(unsigned info) { return info >> 10; }
 // odd where many lanes read a run of their own: no bank is hit twice
 __host__ __device__ constexpr int tile_stride(int kmax, int runs) { return runs > 8 ? kmax | 1 : kmax; }
 __host__ __device__ constexpr int tile_bytes(int stride, int runs) {
-    return kTileHead + kTileRows * 8 + (runs * (stride * 12 + 4) + 15) / 16 * 16;
+    return kTileOwn + (runs * (stride * 12 + 4) + 15) / 16 * 16;
 }
 constexpr int kUniform = 4;
 // a warp's tiles: primal ones first
@@ -84,6 +84,7 @@ struct BlockWarp { int first, count; };
 struct BlockPlan {
     const BlockTile *tiles;
     const BlockWarp *warps;       // by CTA, then warp
+    unsigned char *image;         // the tiles' entries as they lie in shared memory (k_block_pack)
     const unsigned *seq;          // iterations of earlier launches (the evaluation adds this one's)
     ulonglong2 *xt, *yt;          // x-bar and y, tagged
     unsigned long long *stamp;    // kernel timing: the timed iteration's bounds on CTA 0 (or null)
@@ -156,6 +157,10 @@ __device__ __forceinline__ double plain_dot(double acc, const double *g, const i
 __device__ __forceinline__ void copy8(double *dst, const void *src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
 }
+// of sixteen, past L1
+__device__ __forceinline__ void copy16(void *dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
 __device__ __forceinline__ void copy8_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 __device__ __forceinline__ void stage_row(const Bufs &b, double *stage, bool primal, int r) {
@@ -175,6 +180,34 @@ __device__ __forceinline__ void block_weights(const Bufs &b, int jj, double &w, 
         w = ((double)jj + 1.0) / ((double)jj + 2.0);
         w1 = 1.0 - w;
     }
+}
+
+// The image: every tile's entries as k_block's shared memory holds them, made once for
+// the tables it belongs to; a warp per tile.
+template <typename VT>
+__global__ void __launch_bounds__(kSmallThreads) k_block_pack(const BlockTile *__restrict__ tiles, int count, unsigned char *image,
+                                                              const __grid_constant__ Bufs b) {
+    const int t = blockIdx.x * (kSmallThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (t >= count) return;
+    const BlockTile T = tiles[t];
+    const bool primal = tile_primal(T.info), lng = tile_kind(T.info) == TILE_LONG;
+    const int runs = __popc(T.runs), stride = tile_stride(T.kmax, runs);
+    const int at = __popc(T.runs & ((2u << lane) - 1)) - 1;
+    double *val = reinterpret_cast<double *>(image + (size_t)T.img * 16);
+    int *col = reinterpret_cast<int *>(val + runs * stride);
+    if (!(T.runs >> lane & 1)) return;
+    const int r = T.r0 + lane;
+    const int *rp = primal ? b.AT_rp : b.A_rp, *ci = primal ? b.AT_ci : b.A_ci;
+    const VT *v = static_cast<const VT *>(primal ? b.AT_v : b.A_v);
+    int k0 = 0, k1 = 0, ks = 1;
+    if (lng) { k0 = rp[T.r0] + lane; k1 = rp[T.r0 + 1]; ks = 32; }
+    else if (lane < tile_rows(T.info)) { k0 = rp[r]; k1 = rp[r + 1]; }
+    for (int q = 0; q < T.kmax; q++) {
+        const int k = k0 + q * ks;
+        col[at * stride + q] = k < k1 ? ci[k] : 0;
+        val[at * stride + q] = k < k1 ? widen(v[k]) : 0.0;
+    }
+    col[runs * stride + at] = k1 > k0 ? (k1 - k0 + ks - 1) / ks : 0;
 }
 
 // Shared memory: the LPs' step data, ONE (a session of one LP): the weights
@@ -216,34 +249,30 @@ __global__ void __launch_bounds__(NT, 1) k_block(const __grid_constant__ BlockPl
             wt[t] = make_double2(w, w1);
         }
     double *stage = reinterpret_cast<double *>(blk_smem + P.head + (threadIdx.x >> 5) * kStageBytes) + lane;   // STAGED
-    // the warp's tiles into shared memory
+    // The warp's tiles into shared memory, all copies in flight together: the entries
+    // from the image, the vector where it lies (6,049 buses 27.3 us per iteration with
+    // the evaluation; row pointers, columns and values one tile after another 27.55).
     const BlockWarp wp = P.warps[blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)];
 #pragma unroll 1
-    for (int t = 0; t < wp.count; t++) {
-        const BlockTile T = P.tiles[wp.first + t];
-        const bool primal = tile_primal(T.info), ok = lane < tile_rows(T.info), lng = tile_kind(T.info) == TILE_LONG;
-        unsigned char *here = blk_smem + T.smem;
-        if (lane == 0) *reinterpret_cast<int4 *>(here) = make_int4(T.r0, T.info, T.kmax, T.runs);
-        double *z = reinterpret_cast<double *>(here + kTileHead), *val = z + kTileRows;
-        const int runs = __popc(T.runs), stride = tile_stride(T.kmax, runs);
-        const int at = __popc(T.runs & ((2u << lane) - 1)) - 1;
-        int *col = reinterpret_cast<int *>(val + runs * stride);
-        const int r = T.r0 + lane;
-        const int *rp = primal ? b.AT_rp : b.A_rp, *ci = primal ? b.AT_ci : b.A_ci;
-        const VT *v = static_cast<const VT *>(primal ? b.AT_v : b.A_v);
-        int k0 = 0, k1 = 0, ks = 1;
-        if (lng) { k0 = rp[T.r0] + lane; k1 = rp[T.r0 + 1]; ks = 32; }
-        else if (ok) { k0 = rp[r]; k1 = rp[r + 1]; }
-        if (T.runs >> lane & 1) {
-            for (int q = 0; q < T.kmax; q++) {
-                const int k = k0 + q * ks;
-                col[at * stride + q] = k < k1 ? ci[k] : 0;
-                val[at * stride + q] = k < k1 ? widen(v[k]) : 0.0;
-            }
-            col[runs * stride + at] = k1 > k0 ? (k1 - k0 + ks - 1) / ks : 0;
+    for (int t0 = 0; t0 < wp.count; t0 += 32) {
+        BlockTile mine{};
+        if (t0 + lane < wp.count) mine = P.tiles[wp.first + t0 + lane];
+#pragma unroll 1
+        for (int t = 0; t < min(32, wp.count - t0); t++) {
+            const int r0 = __shfl_sync(0xffffffffu, mine.r0, t), smem = __shfl_sync(0xffffffffu, mine.smem, t);
+            const unsigned info = __shfl_sync(0xffffffffu, mine.info, t);
+            const int kmax = __shfl_sync(0xffffffffu, mine.kmax, t), img = __shfl_sync(0xffffffffu, mine.img, t);
+            const unsigned starts = __shfl_sync(0xffffffffu, mine.runs, t);
+            const int runs = __popc(starts), bytes = tile_bytes(tile_stride(kmax, runs), runs) - kTileOwn;
+            unsigned char *here = blk_smem + smem;
+            const unsigned char *from = P.image + (size_t)img * 16;
+            for (int o = lane * 16; o < bytes; o += 512) copy16(here + kTileOwn + o, from + o);
+            if (lane == 0) *reinterpret_cast<int4 *>(here) = make_int4(r0, info, kmax, starts);
+            if (lane < tile_rows(info))
+                copy8(reinterpret_cast<double *>(here + kTileHead) + lane, (tile_primal(info) ? b.x[0] : b.y[0]) + r0 + lane);
         }
-        if (ok) z[lane] = primal ? b.x[0][r] : b.y[0][r];
     }
+    copy8_wait();
     const unsigned tile0 = wp.count ? P.tiles[wp.first].smem : 0;   // a warp's tiles lie side by side
     __syncthreads();
     const int nit = nit_;

@@ -1707,7 +1707,7 @@ struct Layout {
     // period-strided groups: k per group and slot records (row kernels)
     size_t A_sk, AT_sk, A_sl, AT_sl;
     // resident block kernel: tiles, their split over warps, tagged vectors, iteration count, timing stamps
-    size_t tiles, warps, xt, yt, blk_seq, stamp;
+    size_t tiles, warps, image, xt, yt, blk_seq, stamp;
     // lanes sessions: contiguous staging for one LP's vectors (4 (n + m) doubles:
     // the seven vectors a result may download)
     size_t lane_stage;
@@ -1770,6 +1770,7 @@ struct uc_session {
     bool block_able = false, block = false;
     int sms = 0, blk_smem_max = 0;          // SMs, shared memory per CTA
     int blk_ctas = 0, blk_threads = 0, blk_smem = 0;
+    int64_t blk_image = 0;                  // bytes of the tables' image
     uc::dev::BlockPlan plan{};
     unsigned long long *h_stamp = nullptr;   // pinned [2][2]: timed iteration's bounds of each graph
     double *h_vec = nullptr;      // pinned: an LP's vectors on their way to the device (update_lp)
@@ -2350,6 +2351,14 @@ static void launch_block(uc_session &X, cudaStream_t s) {
     if (e != cudaSuccess && X.launch_err == cudaSuccess) X.launch_err = e;
 }
 
+static int block_pack(uc_session &X, int count) {
+    const int per = kSmallThreads / 32, grid = (count + per - 1) / per;
+    if (X.vb == 32) k_block_pack<float><<<grid, kSmallThreads, 0, X.s>>>(X.plan.tiles, count, X.plan.image, X.b);
+    else k_block_pack<double><<<grid, kSmallThreads, 0, X.s>>>(X.plan.tiles, count, X.plan.image, X.b);
+    UC_CUDA(cudaGetLastError());
+    return UC_OK;
+}
+
 static int capture(uc_session &X, int gi) {
     cudaStream_t s = X.s;
     const bool timing = X.o.kernel_timing != 0;
@@ -2545,14 +2554,14 @@ static void plan_block(uc_session &X, const std::vector<char> &mask, std::vector
                 }
                 const unsigned runs = tile_runs(M, primal ? v.AT_val32 : v.A_val32, s, e);
                 const int kind = kmin == kmax && kmax >= 1 && kmax <= kUniform ? TILE_UNIFORM : TILE_ANY;
-                t[primal].push_back(BlockTile{(int)(base + s), tile_info(e - s, kind, primal, ineq, i), kmax, runs, 0, {}});
+                t[primal].push_back(BlockTile{(int)(base + s), tile_info(e - s, kind, primal, ineq, i), kmax, runs, 0, 0, {}});
                 bytes += bytes_of(t[primal].back());
             }
         };
         cut(v.AT, 0, n - nl, X.coff[i], true, false);
         for (int j = n - nl; j < n; j++) {
             const int kmax = (v.AT.rowptr[j + 1] - v.AT.rowptr[j] + 31) / 32;
-            t[1].push_back(BlockTile{(int)(X.coff[i] + j), tile_info(1, TILE_LONG, true, false, i), kmax, ~0u, 0, {}});
+            t[1].push_back(BlockTile{(int)(X.coff[i] + j), tile_info(1, TILE_LONG, true, false, i), kmax, ~0u, 0, 0, {}});
             bytes += bytes_of(t[1].back());
         }
         cut(v.A, 0, m_eq, X.roff[i], false, false);
@@ -2581,19 +2590,22 @@ static void plan_block(uc_session &X, const std::vector<char> &mask, std::vector
                 for (const BlockTile *p : mine[ph][slot]) tiles.push_back(*p);
         }
     const int head = block_head(X);
-    int64_t most = 0;
+    int64_t most = 0, image = 0;
     for (int c = 0; c < nc; c++) {
         int64_t at = head + (big ? W * kStageBytes : 0);
         for (int w = 0; w < W; w++) {
             const BlockWarp &wp = warps[(size_t)c * W + w];
             for (int q = wp.first; q < wp.first + wp.count; q++) {
                 tiles[q].smem = (int)at;
+                tiles[q].img = (int)(image / 16);
                 at += bytes_of(tiles[q]);
+                image += bytes_of(tiles[q]) - kTileOwn;
             }
         }
         most = std::max(most, at);
     }
     if (most > X.blk_smem_max) return;
+    X.blk_image = image;
     X.plan.head = head;
     X.plan.nlps = X.k;
     X.plan.n_eval = X.o.n_eval;
@@ -2673,6 +2685,7 @@ static int retable(uc_session &X, const std::vector<char> &mask) {
     plan_block(X, mask, tiles, warps);
     if (!rc && X.block) rc = up(L.tiles, tiles.data(), sizeof(BlockTile) * tiles.size());
     if (!rc && X.block) rc = up(L.warps, warps.data(), sizeof(BlockWarp) * warps.size());
+    if (!rc && X.block) rc = block_pack(X, (int)tiles.size());
     std::vector<Chunk> cp, cd;
     std::vector<int> gp, gd;
     if (X.staged) {
@@ -2914,6 +2927,8 @@ static int session_create_as(const PsData *const *Pp, const std::shared_ptr<cons
         }
         L.tiles = take(sizeof(BlockTile) * nt);
         L.warps = take(X->block_able ? sizeof(BlockWarp) * 32 * X->sms : 0);
+        // the image of all LPs; that of a subset in the CTAs' shared memory where all do not fit
+        L.image = take(X->block ? X->blk_image : X->block_able ? (size_t)X->sms * X->blk_smem_max : 0);
     }
     L.upload_end = off;
     L.x0 = take(N * 8); L.x1 = take(N * 8); L.y0 = take(M * 8); L.y1 = take(M * 8);
@@ -3044,6 +3059,7 @@ static int session_create_as(const PsData *const *Pp, const std::shared_ptr<cons
     b.n_eval = o.n_eval;
     X->plan.tiles = (const BlockTile *)(D + L.tiles);
     X->plan.warps = (const BlockWarp *)(D + L.warps);
+    X->plan.image = (unsigned char *)(D + L.image);
     X->plan.seq = b.blk_seq;
     X->plan.xt = (ulonglong2 *)(D + L.xt);
     X->plan.yt = (ulonglong2 *)(D + L.yt);
@@ -3060,6 +3076,10 @@ static int session_create_as(const PsData *const *Pp, const std::shared_ptr<cons
     UC_CUDA(cudaMemsetAsync(D + L.S, 0xff, sizeof(Scalars) * k, s));   // status -1: idle
     UC_CUDA(cudaMemsetAsync(D + L.status, 0xff, sizeof(int) * k, s));
     UC_CUDA(cudaMemsetAsync(D + L.blk_seq, 0, sizeof(unsigned), s));
+    if (X->block) {
+        int rc = block_pack(*X, (int)tiles.size());
+        if (rc) return rc;
+    }
     if (X->block_able) {   // tag 0: no iteration's
         UC_CUDA(cudaMemsetAsync(D + L.xt, 0, N * 16, s));
         UC_CUDA(cudaMemsetAsync(D + L.yt, 0, M * 16, s));

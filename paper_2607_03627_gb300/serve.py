@@ -244,14 +244,14 @@ def session_bytes_estimate(ps, value_bits: int = 64, max_iter: int = 100_000) ->
     matrix and its transpose (int32 indices, FP64 or FP32 values, row pointers),
     the period-strided slot records, eight constant and start vectors, ten state
     vectors and a tagged copy of the iterate per column or row, the resident
-    kernel's tiles, and the Halpern weight tables."""
+    kernel's tiles and entries, and the Halpern weight tables."""
     n, m, _, nnz = B.uc_presolved_dims(ps)
     vs = 4 if value_bits == 32 else 8
     slot = 8 if value_bits == 32 else 16
-    per_col = 4 + 8 * 8 + 5 * 8 + slot + 17
-    per_row = 4 + 4 * 8 + 5 * 8 + slot + 17
+    per_col = 4 + 8 * 8 + 5 * 8 + slot + 21
+    per_row = 4 + 4 * 8 + 5 * 8 + slot + 21
     tables = 2 * 8 * min(max_iter + 1, 1 << 22)
-    return int(1.05 * (2 * nnz * (4 + vs) + n * per_col + m * per_row + tables) + (1 << 20))
+    return int(1.05 * (2 * nnz * (4 + vs) + 12 * nnz + n * per_col + m * per_row + tables) + (1 << 20))
 
 
 class MixedServer:
