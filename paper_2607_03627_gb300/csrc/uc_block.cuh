@@ -108,9 +108,9 @@ __device__ __forceinline__ ulonglong2 ld_tagged(const ulonglong2 *p) {
     return w;
 }
 
-// Every wait ends: after so many polls (0.3 to 1 us each) *stalled is set and the
-// caller leaves.
-constexpr unsigned kBlockPolls = 1u << 22;
+// Every wait ends: after so many polls (0.3 to 1 us each, 10 s at least: the grid's last
+// CTA may have to wait for another stream's kernel) *stalled is set and the caller leaves.
+constexpr unsigned kBlockPolls = 1u << 25;
 
 // arrived() + (this lane's entries) . g, in order, N gathers in flight; entry q at
 // q, its column plus add; g tagged and awaited.  ALL: every lane has N entries.  arrived()
