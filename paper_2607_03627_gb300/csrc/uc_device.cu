@@ -1052,8 +1052,8 @@ __device__ __forceinline__ bool differ(double a, double b) { return __double_as_
 // evaluation's time: 6 round trips to L2 for a row of three entries instead of 3)
 template <typename VT, typename At, typename F>
 __device__ __forceinline__ void each_entry(const int *__restrict__ ci, const VT *__restrict__ v, const double *g, At at,
-                                           int k0, int k1, int step, F f) {
-    for (int k = k0; k < k1; k += 4 * step) {
+                                           unsigned k0, unsigned k1, unsigned step, F f) {
+    for (unsigned k = k0; k < k1; k += 4 * step) {   // unsigned: k1 may be close to 2^31
         size_t j[4];
         double a[4], gj[4];
 #pragma unroll
@@ -3544,9 +3544,11 @@ static __device__ __align__(256) double g_kkt_scratch[kNoAllocMaxBlocks * kNoAll
 static __device__ unsigned g_kkt_ended[kNoAllocTickets][kNoAllocMaxBlocks / kNoAllocGroup + 1];
 
 // row . v, entries in order, the loads of four entries in flight together; an
-// FMA step issues only if some lane needs it
+// FMA step issues only if some lane needs it.  A lane whose row has ended stays at its
+// end (k1) while others go on, and indices are unsigned: none passes 2^31 + 3, and a
+// matrix of up to 2^31 - 1 entries is read in bounds.
 __device__ __forceinline__ double csr_dot(const int32_t *__restrict__ ci, const double *__restrict__ av,
-                                          const double *__restrict__ v, int k0, int k1) {
+                                          const double *__restrict__ v, unsigned k0, unsigned k1) {
     double s = 0.0;
     const unsigned lanes = __activemask();
 #pragma unroll 1
@@ -3563,7 +3565,7 @@ __device__ __forceinline__ double csr_dot(const int32_t *__restrict__ ci, const 
             if (!__any_sync(lanes, k0 + q < k1)) break;
             if (k0 + q < k1) s = fma(a[q], g[q], s);
         }
-        k0 += 4;
+        k0 = min(k0 + 4, k1);
     }
     return s;
 }
@@ -3799,7 +3801,8 @@ __global__ void __launch_bounds__(kPwThreads) k_pw_spmv(const int32_t *__restric
                                                         const double *__restrict__ val, int rows, const double *x, double *y,
                                                         double *part, PwState *st, double tol) {
     const int i = blockIdx.x * kPwThreads + threadIdx.x;
-    int k0 = 0, k1 = 0, c[4];
+    unsigned k0 = 0, k1 = 0;   // as in csr_dot: no index passes 2^31 + 3
+    int c[4];
     double a[4], s = 0.0;
     if (i < rows) { k0 = rp[i]; k1 = rp[i + 1]; }
 #pragma unroll
@@ -3817,7 +3820,7 @@ __global__ void __launch_bounds__(kPwThreads) k_pw_spmv(const int32_t *__restric
             if (!__any_sync(0xffffffffu, k0 + q < k1)) break;
             if (k0 + q < k1) s = fma(a[q], g[q], s);
         }
-        k0 += 4;
+        k0 = min(k0 + 4, k1);
 #pragma unroll
         for (int q = 0; q < 4; q++) if (k0 + q < k1) { c[q] = ld_stream(ci + k0 + q); a[q] = ld_stream(val + k0 + q); }
     }
