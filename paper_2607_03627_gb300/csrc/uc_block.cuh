@@ -89,6 +89,7 @@ struct BlockPlan {
     ulonglong2 *xt, *yt;          // x-bar and y, tagged
     unsigned long long *stamp;    // kernel timing: the timed iteration's bounds on CTA 0 (or null)
     int stamp_it, nlps, n_eval, head;   // head: bytes before the warps' staged constants and the tiles
+    unsigned polls;               // a wait's limit
 };
 struct __align__(16) BlockLp { double tau, nsigma; int j, lim, pad[2]; };
 
@@ -108,8 +109,12 @@ __device__ __forceinline__ ulonglong2 ld_tagged(const ulonglong2 *p) {
     return w;
 }
 
-// Every wait ends: after so many polls (0.3 to 1 us each, 10 s at least: the grid's last
-// CTA may have to wait for another stream's kernel) *stalled is set and the caller leaves.
+// Every wait ends: after BlockPlan::polls polls (0.3 to 1 us each) stalled is set and the
+// caller leaves.  The CTAs of a cooperative launch start together, once all of them fit
+// beside what other streams run (40 SMs held for 20 ms: all 152 CTAs start within 1 us
+// of one another after that; two such launches of one CTA per SM run one after the
+// other, whatever their streams' priorities), so another kernel delays the launch and
+// never an element; the limit, 10 s at least, only ends what a defect would let hang.
 constexpr unsigned kBlockPolls = 1u << 25;
 
 // arrived() + (this lane's entries) . g, in order, N gathers in flight; entry q at
@@ -117,7 +122,7 @@ constexpr unsigned kBlockPolls = 1u << 25;
 // is called when the first words are there.
 template <int N, bool ALL, typename F>
 __device__ __forceinline__ double tile_dot(const ulonglong2 *g, unsigned tag, const int *col, const double *val,
-                                           int add, int kmax, int cnt, bool &stalled, F &&arrived) {
+                                           int add, int kmax, int cnt, unsigned polls, bool &stalled, F &&arrived) {
     double acc = 0.0;
     g += add;
 #pragma unroll 1
@@ -134,7 +139,7 @@ __device__ __forceinline__ double tile_dot(const ulonglong2 *g, unsigned tag, co
                     w[q] = ld_tagged(g + col[e + q]);
                 }
             if (__all_sync(0xffffffffu, ready)) break;
-            if (n > kBlockPolls) { stalled = true; return acc; }
+            if (n > polls) { stalled = true; return acc; }
         }
         if (ALL || e == 0) acc = arrived();
 #pragma unroll
@@ -326,11 +331,11 @@ __global__ void __launch_bounds__(NT, 1) k_block(const __grid_constant__ BlockPl
                 if (primal && it == 0) {
                     acc = plain_dot(arrived(), b.y[0], col, val, add, cnt);
                 } else if (tile_kind(T.y) == TILE_UNIFORM) {
-                    if (kmax == 3) acc = tile_dot<3, true>(gt, want, col, val, add, 3, 3, stalled, arrived);
-                    else if (kmax == 2) acc = tile_dot<2, true>(gt, want, col, val, add, 2, 2, stalled, arrived);
-                    else if (kmax == 1) acc = tile_dot<1, true>(gt, want, col, val, add, 1, 1, stalled, arrived);
-                    else acc = tile_dot<4, true>(gt, want, col, val, add, 4, 4, stalled, arrived);
-                } else acc = tile_dot<N, false>(gt, want, col, val, add, kmax, cnt, stalled, arrived);
+                    if (kmax == 3) acc = tile_dot<3, true>(gt, want, col, val, add, 3, 3, P.polls, stalled, arrived);
+                    else if (kmax == 2) acc = tile_dot<2, true>(gt, want, col, val, add, 2, 2, P.polls, stalled, arrived);
+                    else if (kmax == 1) acc = tile_dot<1, true>(gt, want, col, val, add, 1, 1, P.polls, stalled, arrived);
+                    else acc = tile_dot<4, true>(gt, want, col, val, add, 4, 4, P.polls, stalled, arrived);
+                } else acc = tile_dot<N, false>(gt, want, col, val, add, kmax, cnt, P.polls, stalled, arrived);
                 if (kmax == 0) acc = arrived();
                 if (stalled) break;
                 if (lng) {
@@ -392,6 +397,7 @@ __global__ void __launch_bounds__(NT, 1) k_block(const __grid_constant__ BlockPl
         }
         if (stalled) break;
     }
+    copy8_wait();   // a wait that ran out may have left a row's constants in flight
     if (stalled && lane == 0)
         for (int i = 0; i < P.nlps; i++)
             if (b.S[i].status == RUNNING) { b.S[i].status = STALLED; b.status[i] = STALLED; }

@@ -1052,18 +1052,18 @@ __device__ __forceinline__ bool differ(double a, double b) { return __double_as_
 // evaluation's time: 6 round trips to L2 for a row of three entries instead of 3)
 template <typename VT, typename At, typename F>
 __device__ __forceinline__ void each_entry(const int *__restrict__ ci, const VT *__restrict__ v, const double *g, At at,
-                                           unsigned k0, unsigned k1, unsigned step, F f) {
-    for (unsigned k = k0; k < k1; k += 4 * step) {   // unsigned: k1 may be close to 2^31
+                                           unsigned k, unsigned k1, int step, F f) {
+    for (int left = (int)(k1 - k); left > 0; left -= 4 * step, k += 4 * step) {   // k1 may be close to 2^31
         size_t j[4];
         double a[4], gj[4];
 #pragma unroll
         for (int q = 0; q < 4; q++)
-            if (k + q * step < k1) { j[q] = at(__ldg(ci + k + q * step)); a[q] = widen(__ldg(v + k + q * step)); }
+            if (q * step < left) { j[q] = at(__ldg(ci + k + q * step)); a[q] = widen(__ldg(v + k + q * step)); }
 #pragma unroll
-        for (int q = 0; q < 4; q++) if (k + q * step < k1) gj[q] = g[j[q]];
+        for (int q = 0; q < 4; q++) if (q * step < left) gj[q] = g[j[q]];
 #pragma unroll
         for (int q = 0; q < 4; q++) {
-            if (k + q * step >= k1) break;
+            if (q * step >= left) break;
             f(a[q], gj[q], j[q]);
         }
     }
@@ -3702,20 +3702,21 @@ __global__ void __launch_bounds__(kThreads, kNoAllocCtas) k_kkt_noalloc(uc_devic
             const double d = ld_stream(lp.Dc + j), xj = __ldg(x + j);
             const double lm = cj - csr_dot(lp.AT_colidx, lp.AT_val, y, k0, k1);
             const bool lf = is_fin(lj), uf = is_fin(uj);
-            // reduced cost inside the cone the bounds allow (lp_j) and the rest, rd = lm - lp_j,
-            // by sign tests; where lm is not finite by the subtraction (inf - inf is NaN)
-            double lp_j = lf && uf ? lm : lf ? pos_part(lm) : uf ? neg_part(lm) : 0.0;
-            double rd = lf && uf ? 0.0 : lf ? neg_part(lm) : uf ? pos_part(lm) : lm;
-            const bool fin = is_fin(lm);
-            if (!fin) {
-                if (is_nan(lm)) lp_j = 0.0;
-                rd = lm - lp_j;
+            // reduced cost inside the cone the bounds allow (lp_j) and the rest (rd = lm - lp_j):
+            // by sign tests, but inf - inf, the rest of an infinity inside the cone, is NaN
+            double rd, lp_j = 0.0;
+            if (is_nan(lm)) {
+                rd = lm;
+            } else {
+                lp_j = lf && uf ? lm : lf ? pos_part(lm) : uf ? neg_part(lm) : 0.0;
+                rd = lf && uf ? 0.0 : lf ? neg_part(lm) : uf ? pos_part(lm) : lm;
+                if (!is_fin(lp_j)) rd = __longlong_as_double(0x7ff8000000000000LL);
             }
             const double bound = is_neg(lp_j) ? (uf ? uj : 0.0) : (lf ? lj : 0.0);
             const unsigned lanes = __activemask();
             if (__any_sync(lanes, mag_bits(rd) != 0)) a0 = fma(rd, rd, a0);
             if (__any_sync(lanes, mag_bits(cj) != 0 || !is_fin(xj))) a1 = fma(cj, xj, a1);
-            if (__any_sync(lanes, !fin || (mag_bits(bound) != 0 && mag_bits(lp_j) != 0))) a2 = fma(bound, lp_j, a2);
+            if (__any_sync(lanes, !is_fin(lp_j) || (mag_bits(bound) != 0 && mag_bits(lp_j) != 0))) a2 = fma(bound, lp_j, a2);
             quot.add(rd, d);
         }
     }
