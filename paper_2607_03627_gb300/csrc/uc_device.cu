@@ -3065,6 +3065,7 @@ static int session_create_as(const PsData *const *Pp, const std::shared_ptr<cons
     X->plan.yt = (ulonglong2 *)(D + L.yt);
     X->plan.stamp = o.kernel_timing ? (unsigned long long *)(D + L.stamp) : nullptr;
     X->plan.stamp_it = o.n_eval / 2;
+    X->plan.polls = kBlockPolls;
     b.S = (Scalars *)(D + L.S);
     b.status = (int *)(D + L.status);
     X->dsp = (const Seg *)(D + L.segs_p); X->dsd = (const Seg *)(D + L.segs_d);
@@ -4064,6 +4065,14 @@ int uc_session_update_lp(uc_session *s, int i, const uc_presolved *ps) {
         set_error("out of host memory");
         return UC_ENOMEM;
     }
+}
+
+int uc_session_wait_limit(uc_session *s, unsigned polls) {
+    if (!s) { set_error("uc_session_wait_limit: null session"); return UC_EINVAL; }
+    UC_CUDA(cudaStreamSynchronize(s->s));
+    s->plan.polls = polls;
+    const std::vector<char> tabled = s->tabled;
+    return dev::retable(*s, tabled);   // the graphs hold the plan
 }
 
 size_t uc_session_device_bytes(const uc_session *s) { return s ? s->bytes : 0; }

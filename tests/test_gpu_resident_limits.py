@@ -1,0 +1,55 @@
+"""The resident block kernel at its limits: a wait that runs out."""
+import ctypes
+
+import numpy as np
+import pytest
+
+import ucgen
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2607_03627_gb300 as pkg
+    pkg.build()
+    from paper_2607_03627_gb300 import binding
+    return binding
+
+
+def _presolved(B, seed, buses, periods, units, **kw):
+    return B.uc_presolve(B.uc_build_lp(ucgen.make_problem(
+        seed, B=buses, L=int(1.32 * buses), G=units, T=periods, lo=0.4, hi=0.8, noise=0.05, zero_pmin_frac=0.1)),
+        power_max_iter=20, **kw)
+
+
+def _same(B, ra, rb, ps):
+    n, m, _, _ = B.uc_presolved_dims(ps)
+    sa, sb = B.uc_get_stats(ra), B.uc_get_stats(rb)
+    for key in ("status", "iters", "restarts", "evals", "omega", "rel_primal", "rel_dual", "rel_gap"):
+        assert sa[key] == sb[key], (key, sa[key], sb[key])
+    for which in (0, 1, 2):
+        for a, b in zip(B.uc_get_iterate(ra, which, n, m), B.uc_get_iterate(rb, which, n, m)):
+            np.testing.assert_array_equal(a, b)
+
+
+def test_a_wait_that_runs_out_is_an_error_status_and_the_session_goes_on(B):
+    # every wait gives up after its second look: the kernel ends, the LP is reported as
+    # failed, and with the usual limit the session solves as ever
+    ps = _presolved(B, 6, 300, 24, 36)
+    limit = B.lib.uc_session_wait_limit
+    limit.argtypes, limit.restype = [ctypes.c_void_p, ctypes.c_uint], ctypes.c_int
+    s = B.Session([ps], tol=0.0, max_iter=640)
+    assert limit(s.ptr, 0) == B.UC_OK
+    s.reset(-1)
+    s.run()
+    _, rc = s.result(0)
+    assert rc == B.UC_ECUDA and b"stopped waiting" in B.lib.uc_last_error()
+    assert limit(s.ptr, 1 << 25) == B.UC_OK
+    s.reset(-1)
+    s.run()
+    _same(B, B.uc_solve(ps, tol=0.0, max_iter=640, spmv_kernel=1)[0], s.result(0)[0], ps)
+    s.close()
