@@ -3064,7 +3064,7 @@ static int session_create_as(const PsData *const *Pp, const std::shared_ptr<cons
     X->plan.xt = (ulonglong2 *)(D + L.xt);
     X->plan.yt = (ulonglong2 *)(D + L.yt);
     X->plan.stamp = o.kernel_timing ? (unsigned long long *)(D + L.stamp) : nullptr;
-    X->plan.stamp_it = o.n_eval / 2;
+    X->plan.stamp_it = o.n_eval / 2 - 1;   // its end is the next iteration's start
     X->plan.polls = kBlockPolls;
     b.S = (Scalars *)(D + L.S);
     b.status = (int *)(D + L.status);

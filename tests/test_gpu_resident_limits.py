@@ -1,4 +1,5 @@
-"""The resident block kernel at its limits: a wait that runs out."""
+"""The resident block kernel at its limits: a wait that runs out, blocks too short
+for the timed iteration."""
 import ctypes
 
 import numpy as np
@@ -53,3 +54,18 @@ def test_a_wait_that_runs_out_is_an_error_status_and_the_session_goes_on(B):
     s.run()
     _same(B, B.uc_solve(ps, tol=0.0, max_iter=640, spmv_kernel=1)[0], s.result(0)[0], ps)
     s.close()
+
+
+# every block of n_eval iterations times one of them; a block that the budget ends
+# before it times none
+@pytest.mark.parametrize("n_eval,budget,timed", [(2, 64, True), (4, 64, True), (64, 640, True), (64, 20, False)])
+def test_kernel_timing_of_short_blocks(B, n_eval, budget, timed):
+    ps = _presolved(B, 1, 60, 24, 8)
+    st = B.uc_get_stats(B.uc_solve(ps, tol=0.0, max_iter=budget, n_eval=n_eval, kernel_timing=True)[0])
+    assert st["kernel_launches"] < budget * 5            # the resident kernel: five launches a block
+    if not timed:
+        assert st["timed_launches"] == 0
+        return
+    # the last block ends the solve and is not read
+    assert budget // n_eval - 2 <= st["timed_launches"] <= budget // n_eval
+    assert 0 < st["primal_kernel_ms"] + st["dual_kernel_ms"] < 1
