@@ -3575,11 +3575,10 @@ __device__ __forceinline__ double csr_dot(const int32_t *__restrict__ ci, const 
 // much as an FMA, and the kernel is bound by that pipe.
 __device__ __forceinline__ unsigned long long mag_bits(double v) { return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffULL; }
 __device__ __forceinline__ bool is_nan(double v) { return mag_bits(v) > 0x7ff0000000000000ULL; }
-// |v| cut to FP32 (relative error < 2^-23), or NaN outside [2^-62, 2^62): quotients
-// of two are normal FP32 values, whose relative error is as small
+// |v| cut to FP32 (relative error < 2^-23), or NaN outside [2^-100, 2^100)
 __device__ __forceinline__ float mag_float(double v) {
     const unsigned hi = (unsigned)__double2hiint(v) & 0x7fffffffu, lo = (unsigned)__double2loint(v);
-    if (hi - ((1023u - 62u) << 20) >= (124u << 20)) return __int_as_float(0x7fc00000);
+    if (hi - ((1023u - 100u) << 20) >= (200u << 20)) return __int_as_float(0x7fc00000);
     return __uint_as_float(((hi - ((1023u - 127u) << 20)) << 3) | (lo >> 29));
 }
 
