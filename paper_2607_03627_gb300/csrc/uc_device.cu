@@ -3702,21 +3702,24 @@ __global__ void __launch_bounds__(kThreads, kNoAllocCtas) k_kkt_noalloc(uc_devic
             const double d = ld_stream(lp.Dc + j), xj = __ldg(x + j);
             const double lm = cj - csr_dot(lp.AT_colidx, lp.AT_val, y, k0, k1);
             const bool lf = is_fin(lj), uf = is_fin(uj);
-            // reduced cost inside the cone the bounds allow (lp_j) and the rest (rd = lm - lp_j):
-            // by sign tests, but inf - inf, the rest of an infinity inside the cone, is NaN
+            // reduced cost inside the cone the bounds allow (lp_j) and the rest, rd = lm - lp_j,
+            // by sign tests; of an lm that is not finite by the subtraction (inf - inf is NaN)
             double rd, lp_j = 0.0;
-            if (is_nan(lm)) {
-                rd = lm;
+            if (lf && uf) {
+                if (!is_nan(lm)) lp_j = lm;
+                rd = is_fin(lm) ? 0.0 : __longlong_as_double(0x7ff8000000000000LL);
+            } else if (!is_fin(lm)) {
+                if (!is_nan(lm)) lp_j = lf ? pos_part(lm) : uf ? neg_part(lm) : 0.0;
+                rd = lm - lp_j;
             } else {
-                lp_j = lf && uf ? lm : lf ? pos_part(lm) : uf ? neg_part(lm) : 0.0;
-                rd = lf && uf ? 0.0 : lf ? neg_part(lm) : uf ? pos_part(lm) : lm;
-                if (!is_fin(lp_j)) rd = __longlong_as_double(0x7ff8000000000000LL);
+                lp_j = lf ? pos_part(lm) : uf ? neg_part(lm) : 0.0;
+                rd = lf ? neg_part(lm) : uf ? pos_part(lm) : lm;
             }
             const double bound = is_neg(lp_j) ? (uf ? uj : 0.0) : (lf ? lj : 0.0);
             const unsigned lanes = __activemask();
             if (__any_sync(lanes, mag_bits(rd) != 0)) a0 = fma(rd, rd, a0);
             if (__any_sync(lanes, mag_bits(cj) != 0 || !is_fin(xj))) a1 = fma(cj, xj, a1);
-            if (__any_sync(lanes, !is_fin(lp_j) || (mag_bits(bound) != 0 && mag_bits(lp_j) != 0))) a2 = fma(bound, lp_j, a2);
+            if (__any_sync(lanes, mag_bits(lp_j) != 0 && (mag_bits(bound) != 0 || !is_fin(lp_j)))) a2 = fma(bound, lp_j, a2);
             quot.add(rd, d);
         }
     }
