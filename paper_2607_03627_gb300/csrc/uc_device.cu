@@ -2927,10 +2927,10 @@ static int session_create_as(const PsData *const *Pp, const std::shared_ptr<cons
         }
         L.tiles = take(sizeof(BlockTile) * nt);
         L.warps = take(X->block_able ? sizeof(BlockWarp) * 32 * X->sms : 0);
-        // the image of all LPs; that of a subset in the CTAs' shared memory where all do not fit
-        L.image = take(X->block ? X->blk_image : X->block_able ? (size_t)X->sms * X->blk_smem_max : 0);
     }
     L.upload_end = off;
+    // packed on the device: the image of all LPs; that of a subset in the CTAs' shared memory where all do not fit
+    L.image = take(X->block ? X->blk_image : X->block_able ? (size_t)X->sms * X->blk_smem_max : 0);
     L.x0 = take(N * 8); L.x1 = take(N * 8); L.y0 = take(M * 8); L.y1 = take(M * 8);
     L.xsum = take(N * 8); L.ysum = take(M * 8); L.xa = take(N * 8); L.ya = take(M * 8);
     L.xret = take(N * 8); L.yret = take(M * 8);

@@ -1,5 +1,5 @@
 """The resident block kernel at its limits: a wait that runs out, blocks too short
-for the timed iteration."""
+for the timed iteration, what a session uploads."""
 import ctypes
 
 import numpy as np
@@ -69,3 +69,12 @@ def test_kernel_timing_of_short_blocks(B, n_eval, budget, timed):
     # the last block ends the solve and is not read
     assert budget // n_eval - 2 <= st["timed_launches"] <= budget // n_eval
     assert 0 < st["primal_kernel_ms"] + st["dual_kernel_ms"] < 1
+
+
+def test_upload_has_no_packed_entries(B):
+    # against a session on the row kernels (n_eval above the resident kernel's limit): only
+    # the tiles (32 bytes per 32 rows or columns of a kind) and the warps' lists come along
+    ps = _presolved(B, 2, 300, 24, 36)
+    n, m, _, _ = B.uc_presolved_dims(ps)
+    sent = [B.uc_get_stats(B.uc_solve(ps, tol=0.0, max_iter=64, n_eval=e)[0])["h2d_bytes"] for e in (64, 1026)]
+    assert 0 < sent[0] - sent[1] < 2 * (n + m) + 64 * 1024
