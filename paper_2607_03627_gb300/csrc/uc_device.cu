@@ -2721,10 +2721,13 @@ static int retable(uc_session &X, const std::vector<char> &mask) {
 
 static bool live_status(int st) { return st == RUNNING || st == NEEDS_INIT; }
 
-// split: a lanes session may store its LPs one after another (see below)
+// resident: the session may take memory for the resident kernel, a lanes session then
+// storing its LPs one after another (see below); set to whether it did
 static int session_create_as(const PsData *const *Pp, const std::shared_ptr<const PsData> *owners, int k,
-                             const uc_solve_opts &o, cudaStream_t user_stream, bool split, uc_session **out) {
+                             const uc_solve_opts &o, cudaStream_t user_stream, bool &resident, uc_session **out) {
     *out = nullptr;
+    const bool may = resident;
+    resident = false;
     if (k < 1) { set_error("need at least one LP"); return UC_EINVAL; }
     if (o.n_eval < 2 || (o.n_eval & 1)) { set_error("n_eval must be even and >= 2"); return UC_EINVAL; }
     if (o.max_iter < 0) { set_error("max_iter must be >= 0"); return UC_EINVAL; }
@@ -2814,9 +2817,9 @@ static int session_create_as(const PsData *const *Pp, const std::shared_ptr<cons
         // row indices are also stored shifted left by one bit in the evaluation table
         return X->M < (1LL << 30) && X->N < INT32_MAX && X->Z < INT32_MAX;
     };
-    if (!lay_out(o.lanes && !split)) {
-        split = false;
-        if (!o.lanes || !lay_out(true)) { set_error("batch too large for int32 indices"); return UC_EINVAL; }
+    if (!lay_out(o.lanes && !may) && (!o.lanes || !lay_out(true))) {
+        set_error("batch too large for int32 indices");
+        return UC_EINVAL;
     }
 
     X->rpt.assign(k, 1);
@@ -2854,7 +2857,7 @@ static int session_create_as(const PsData *const *Pp, const std::shared_ptr<cons
         UC_CUDA(cudaDeviceGetAttribute(&X->sms, cudaDevAttrMultiProcessorCount, dev));
         UC_CUDA(cudaDeviceGetAttribute(&X->blk_smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
         X->blk_smem_max -= 1024;   // the kernel's static part
-        X->block_able = coop && o.spmv_kernel == 0 && X->algo == ALG_HALPERN && X->K == 1 && k <= kBlockMaxLps &&
+        X->block_able = may && coop && o.spmv_kernel == 0 && X->algo == ALG_HALPERN && X->K == 1 && k <= kBlockMaxLps &&
                         o.n_eval <= kBlockMaxEval;
         if (X->block_able)
             for (int nt : {kSmallThreads, kMidThreads, kBigThreads})
@@ -2871,6 +2874,7 @@ static int session_create_as(const PsData *const *Pp, const std::shared_ptr<cons
         X->block_able = false;
         X->cta = 128;   // the lanes kernels are built for 128-thread CTAs
     }
+    resident = X->block_able;
     const int64_t M = X->M, N = X->N, Z = X->Z;
     // CTA tables for every LP (their sizes are the capacities of the device tables)
     std::vector<Seg> sp, sd, se, sa;
@@ -3369,9 +3373,14 @@ static int session_result(uc_session &X, int i, uc_result **out) {
 
 static int session_create(const PsData *const *Pp, const std::shared_ptr<const PsData> *owners, int k,
                           const uc_solve_opts &o, cudaStream_t user_stream, uc_session **out) {
-    int rc = session_create_as(Pp, owners, k, o, user_stream, true, out);
-    // the interleaved layout holds the matrix once
-    if (rc == UC_ENOMEM && o.lanes) rc = session_create_as(Pp, owners, k, o, user_stream, false, out);
+    bool resident = true;
+    int rc = session_create_as(Pp, owners, k, o, user_stream, resident, out);
+    // the row kernels need 16 bytes per row and column and the image less (9 MB of 78 at
+    // 391 k rows and columns), the interleaved layout holds the matrix once
+    if (rc == UC_ENOMEM && resident) {
+        resident = false;
+        rc = session_create_as(Pp, owners, k, o, user_stream, resident, out);
+    }
     return rc;
 }
 

@@ -1,5 +1,6 @@
 """The resident block kernel at its limits: a wait that runs out, blocks too short
-for the timed iteration, what a session uploads."""
+for the timed iteration, what a session uploads,
+sessions that device memory holds only without it."""
 import ctypes
 
 import numpy as np
@@ -78,3 +79,39 @@ def test_upload_has_no_packed_entries(B):
     n, m, _, _ = B.uc_presolved_dims(ps)
     sent = [B.uc_get_stats(B.uc_solve(ps, tol=0.0, max_iter=64, n_eval=e)[0])["h2d_bytes"] for e in (64, 1026)]
     assert 0 < sent[0] - sent[1] < 2 * (n + m) + 64 * 1024
+
+
+# device memory for the row kernels' session but not for the resident kernel's: the
+# session runs on the row kernels; for less: refused as ever
+@pytest.mark.parametrize("kind", ["one", "batch", "lanes"])
+def test_session_that_fits_only_without_the_resident_kernel(B, monkeypatch, kind):
+    base = ucgen.make_problem(5, B=60, L=79, G=8, T=24, lo=0.4, hi=0.8, noise=0.05, zero_pmin_frac=0.1)
+    ps0 = B.uc_presolve(B.uc_build_lp(base), power_max_iter=20)
+    pss, kw = [ps0], dict(tol=0.0, max_iter=130)
+    if kind == "batch":
+        pss = [ps0, _presolved(B, 7, 40, 24, 5), _presolved(B, 8, 30, 5, 4)]
+    if kind == "lanes":
+        pss = [B.uc_presolve_reuse(ps0, B.uc_build_lp(ucgen.served_request(base, 5, r))) for r in range(2)]
+        kw["lanes"] = True
+    rows = B.Session(pss, **dict(kw, n_eval=1026))
+    limit = rows.device_bytes()
+    rows.close()
+
+    class Limited(B._TorchAllocator):
+        def _alloc(self, nbytes, stream, ctx):
+            return super()._alloc(nbytes, stream, ctx) if nbytes <= self.limit else None
+    small = Limited()
+    B._torch_stream_and_allocator()
+    monkeypatch.setattr(B, "_allocator", small)
+    small.limit = limit
+    s = B.Session(pss, **kw)
+    assert s.device_bytes() == limit
+    s.reset(-1)
+    s.run()
+    for i, ps in enumerate(pss):
+        small.limit = 1 << 40
+        _same(B, B.uc_solve(ps, spmv_kernel=1, tol=0.0, max_iter=130)[0], s.result(i)[0], ps)
+    s.close()
+    small.limit = limit - 1
+    with pytest.raises(B.UCError, match="allocator returned NULL"):
+        B.Session(pss, **kw)
