@@ -46,7 +46,7 @@ constexpr int kMidThreads = 768, kMidN = 4;
 constexpr int kBigThreads = 896, kBigN = 3;
 constexpr int kBigTiles = 5;
 constexpr int kBlockMaxLps = 64;       // per-LP step data in shared memory
-constexpr int kBlockMaxEval = 1024;    // one LP: the weights of a block's iterations in shared memory
+constexpr int kBlockMaxEval = UC_RESIDENT_MAX_EVAL;   // one LP: the weights of a block's iterations in shared memory
 
 // A tile: rows [r0, r0 + rows) of A^T or A.  In shared memory: the descriptor's
 // first 16 bytes, the rows' own vector (primal x-bar, dual y), then the entries as

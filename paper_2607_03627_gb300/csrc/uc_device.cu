@@ -3605,7 +3605,10 @@ struct MaxQuotient {
         e2 *= mag_float(r2);
         if (!(e2 < e * 0.99999f)) {
             if (e2 > e * 1.00001f && e2 >= 0.0f && !is_neg(d2)) { r = r2; d = d2; e = e2; }
-            else mx = nnmax(mx, fabs(r2) / d2);
+            else {   // a NaN that the device made has its sign set, which nnmax would take for less than zero
+                const double t = fabs(r2) / d2;
+                mx = nnmax(mx, is_nan(t) ? __longlong_as_double(0x7ff8000000000000LL) : t);
+            }
         }
     }
     __device__ __forceinline__ double finish(int *best) {

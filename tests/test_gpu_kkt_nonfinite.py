@@ -97,3 +97,20 @@ def test_infinite_x_or_y_beside_a_cost(B, value, cost, where):
         y[m - 1], q[m - 1] = value, cost     # no column reads the last rows
     args = (c, np.zeros(n), np.full(n, np.inf), np.ones(n), q, np.ones(m), 520, x, y, np.ones(n))
     _check(_call(B, *args), _want(*args))
+
+
+# a NaN with its sign set, as the device makes of inf - inf, wins the largest residual too
+@pytest.mark.parametrize("sign", [0x7ff8 << 48, 0xfff8 << 48])
+@pytest.mark.parametrize("where", ["x", "y"])
+def test_nan_of_either_sign_wins_the_largest_residual(B, sign, where):
+    n, m, j = 300, 300, 131
+    nan = np.array([sign], np.uint64).view(np.float64)[0]
+    gen = np.random.default_rng(3)
+    x, y, q = np.zeros(n), gen.random(m), gen.random(m)
+    if where == "y":
+        y[j] = nan
+    else:
+        q[j] = nan          # A has no entries: the row's residual is -q
+    args = (gen.random(n), np.full(n, -np.inf), np.full(n, np.inf), np.ones(n), q, np.ones(m), m, x, y, np.ones(n))
+    got = _call(B, *args)
+    assert np.isnan(got[1 if where == "y" else 0]) and np.isnan(got[3])
