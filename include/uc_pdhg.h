@@ -45,7 +45,11 @@ extern "C" {
 #define UC_ETIMEOUT (-6)     /* timeout_ms elapsed (result valid, last iterate) */
 #define UC_ENUMERIC (-7)     /* NaN/Inf in the iterates */
 #define UC_ECANCELLED (-8)   /* opts.cancel was set (result valid, last iterate) */
-#define UC_ECUDA (-9)        /* a CUDA runtime call failed */
+#define UC_ECUDA (-9)        /* a CUDA runtime call failed, or an iteration kernel's wait for its own
+                                data ran out (never on a working device) */
+
+/* Largest n_eval with which a session may run the resident kernel (uc_solve_opts.spmv_kernel). */
+#define UC_RESIDENT_MAX_EVAL 1024
 
 typedef struct uc_lp uc_lp;
 typedef struct uc_presolved uc_presolved;
@@ -117,7 +121,8 @@ typedef struct {
     double tol_rel_kkt;          /* relative KKT tolerance (default 1e-4, Sec. II-D) */
     double tol_abs_feas;         /* reported absolute feasibility threshold (default 1e-5) */
     int max_iter;                /* iteration limit (default 100000, Sec. II-D) */
-    int n_eval;                  /* iterations between KKT / restart evaluations (default 64, even) */
+    int n_eval;                  /* iterations between KKT / restart evaluations (default 64, even;
+                                    above UC_RESIDENT_MAX_EVAL: row kernels, see spmv_kernel) */
     int use_graph;               /* 1: replay CUDA graphs of n_eval iterations (default 1) */
     int kernel_timing;           /* 1: time the primal and dual kernel of the middle iteration of every
                                     replay with events (graph path only).  Where the resident kernel
@@ -141,10 +146,13 @@ typedef struct {
                                     rows and vectors into shared memory ahead of use (Halpern only,
                                     rows of at most 640 entries, else UC_EINVAL).  The strided slots
                                     are not used by shared-matrix (lanes) sessions.  With 0 and the
-                                    Halpern algorithm, a session (of up to 64 LPs) whose matrix and
-                                    vectors fit into the SMs' shared memory runs all iterations between
-                                    two evaluations in one cooperative launch instead; cta_rows,
-                                    rows_per_thread and no_pdl do not apply to it.  All variants give
+                                    Halpern algorithm, a session (of up to 64 LPs, n_eval at most
+                                    UC_RESIDENT_MAX_EVAL) whose matrix and vectors fit into the SMs'
+                                    shared memory runs all iterations between two evaluations in one
+                                    cooperative launch of up to one CTA per SM instead, if device memory
+                                    holds its tables too; cta_rows, rows_per_thread and no_pdl do not
+                                    apply to it.  Beside other streams' work it starts when all its CTAs
+                                    fit at once and waits until then.  All variants give
                                     identical iterates. */
     int cta_rows;                /* threads per CTA of the iteration kernels: 0 (default 128), 128,
                                     256 or 512; results do not depend on it (tuning knob) */

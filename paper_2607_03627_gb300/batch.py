@@ -4,7 +4,7 @@ All LPs are packed block-diagonally into one session, so every PDHG iteration
 is one primal and one dual launch for the whole batch (captured in a CUDA
 graph); each LP keeps its own step sizes, restarts and stopping test, and the
 session drops finished LPs from its launch tables as the batch shrinks.  The
-row split of each LP comes from the autotuner, per size bucket.
+row split of each LP comes from the autotuner, per size bucket and batch size.
 """
 from __future__ import annotations
 
@@ -34,7 +34,8 @@ def solve_batch(pss, tol: float = 1e-4, max_iter: int = 100_000, tuner: Tuner | 
         for p in pss:
             b = bucket_of(B.uc_presolved_dims(p)[3])
             rep.setdefault(b, p)
-        chosen = {b: tuner.choose(p, value_bits) for b, p in rep.items()}
+        total = sum(B.uc_presolved_dims(p)[3] for p in pss)
+        chosen = {b: tuner.choose(p, value_bits, total) for b, p in rep.items()}
         rpts = [chosen[bucket_of(B.uc_presolved_dims(p)[3])] for p in pss]
     import torch
     t0 = time.perf_counter()

@@ -18,6 +18,7 @@ LIB_PATH = os.path.join(_HERE, "libucpdhg.so")
 
 UC_OK, UC_EINVAL, UC_ENOMEM, UC_EINFEASIBLE, UC_EUNBOUNDED = 0, -1, -2, -3, -4
 UC_EITERLIMIT, UC_ETIMEOUT, UC_ENUMERIC, UC_ECANCELLED, UC_ECUDA = -5, -6, -7, -8, -9
+UC_RESIDENT_MAX_EVAL = 1024
 STATUS_NAMES = {0: "optimal", -1: "invalid", -2: "out_of_memory", -3: "infeasible",
                 -4: "unbounded", -5: "iteration_limit", -6: "timeout", -7: "numeric",
                 -8: "cancelled", -9: "cuda_error"}
