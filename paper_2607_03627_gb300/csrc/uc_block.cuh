@@ -62,7 +62,8 @@ struct __align__(16) BlockTile {
     unsigned info;   // see tile_info
     int kmax;
     unsigned runs;
-    int smem, img, pad[2];   // where it is: byte in shared memory, 16-byte unit of the image
+    int smem, img;           // where it is: byte in shared memory, 16-byte unit of the image
+    int bytes, pad;          // in shared memory
 };
 constexpr int kTileHead = 16, kTileOwn = kTileHead + kTileRows * 8;   // before the entries
 __host__ __device__ constexpr unsigned tile_info(int rows, int kind, bool primal, bool ineq, int lp) {

@@ -26,6 +26,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <array>
 #include <atomic>
 #include <chrono>
 #include <climits>
@@ -1772,6 +1773,7 @@ struct uc_session {
     int blk_ctas = 0, blk_threads = 0, blk_smem = 0;
     int64_t blk_image = 0;                  // bytes of the tables' image
     uc::dev::BlockPlan plan{};
+    std::vector<std::array<std::vector<uc::dev::BlockTile>, 2>> cut;   // each LP's tiles, dual and primal (plan_block)
     unsigned long long *h_stamp = nullptr;   // pinned [2][2]: timed iteration's bounds of each graph
     double *h_vec = nullptr;      // pinned: an LP's vectors on their way to the device (update_lp)
     // staged iteration kernels
@@ -2523,6 +2525,40 @@ static unsigned tile_runs(const Csr &M, const std::vector<float> &v32, int a, in
     return runs;
 }
 
+static bool tile_before(const BlockTile &a, const BlockTile &b) {
+    return a.kmax != b.kmax ? a.kmax > b.kmax : a.bytes > b.bytes;
+}
+
+// Tiles of LP i, primal and dual, the longest rows first, then the most bytes; cut once
+// for a session, since an LP's matrix stays.
+static void cut_tiles(uc_session &X, int i) {
+    const PsData &v = *X.Pd[i];
+    const int n = v.n(), m = v.m(), nl = v.long_cols, m_eq = X.m_eq[i];
+    auto add = [&](int r0, unsigned info, int kmax, unsigned runs) {
+        const int count = __builtin_popcount(runs);
+        X.cut[i][tile_primal(info)].push_back(BlockTile{r0, info, kmax, runs, 0, 0, tile_bytes(tile_stride(kmax, count), count), 0});
+    };
+    auto cut = [&](const Csr &M, int a, int b, int64_t base, bool primal, bool ineq) {
+        for (int s = a; s < b; s += kTileRows) {
+            const int e = std::min(b, s + kTileRows);
+            int kmax = 0, kmin = INT_MAX;
+            for (int r = s; r < e; r++) {
+                kmax = std::max(kmax, M.rowptr[r + 1] - M.rowptr[r]);
+                kmin = std::min(kmin, M.rowptr[r + 1] - M.rowptr[r]);
+            }
+            const unsigned runs = tile_runs(M, primal ? v.AT_val32 : v.A_val32, s, e);
+            const int kind = kmin == kmax && kmax >= 1 && kmax <= kUniform ? TILE_UNIFORM : TILE_ANY;
+            add((int)(base + s), tile_info(e - s, kind, primal, ineq, i), kmax, runs);
+        }
+    };
+    cut(v.AT, 0, n - nl, X.coff[i], true, false);
+    for (int j = n - nl; j < n; j++)
+        add((int)(X.coff[i] + j), tile_info(1, TILE_LONG, true, false, i), (v.AT.rowptr[j + 1] - v.AT.rowptr[j] + 31) / 32, ~0u);
+    cut(v.A, 0, m_eq, X.roff[i], false, false);
+    cut(v.A, m_eq, m, X.roff[i], false, true);
+    for (auto &t : X.cut[i]) std::stable_sort(t.begin(), t.end(), tile_before);
+}
+
 // Tiles of the resident block kernel for the LPs in `mask`, dealt to the warps of
 // at most one CTA per SM: primal tiles, longest rows first, to the warps in turn
 // over the CTAs, dual tiles in turn from the last warp back, so that a warp has
@@ -2534,39 +2570,26 @@ static void plan_block(uc_session &X, const std::vector<char> &mask, std::vector
     warps.clear();
     X.block = false;
     if (!X.block_able) return;
+    X.cut.resize(X.k);
     std::vector<BlockTile> t[2];   // dual, primal
-    auto bytes_of = [](const BlockTile &T) {
-        const int runs = __builtin_popcount(T.runs);
-        return tile_bytes(tile_stride(T.kmax, runs), runs);
-    };
     int64_t bytes = 0;
     for (int i = 0; i < X.k; i++) {
         if (!mask[i]) continue;
-        const PsData &v = *X.Pd[i];
-        const int n = v.n(), m = v.m(), nl = v.long_cols, m_eq = X.m_eq[i];
-        auto cut = [&](const Csr &M, int a, int b, int64_t base, bool primal, bool ineq) {
-            for (int s = a; s < b; s += kTileRows) {
-                const int e = std::min(b, s + kTileRows);
-                int kmax = 0, kmin = INT_MAX;
-                for (int r = s; r < e; r++) {
-                    kmax = std::max(kmax, M.rowptr[r + 1] - M.rowptr[r]);
-                    kmin = std::min(kmin, M.rowptr[r + 1] - M.rowptr[r]);
-                }
-                const unsigned runs = tile_runs(M, primal ? v.AT_val32 : v.A_val32, s, e);
-                const int kind = kmin == kmax && kmax >= 1 && kmax <= kUniform ? TILE_UNIFORM : TILE_ANY;
-                t[primal].push_back(BlockTile{(int)(base + s), tile_info(e - s, kind, primal, ineq, i), kmax, runs, 0, 0, {}});
-                bytes += bytes_of(t[primal].back());
-            }
-        };
-        cut(v.AT, 0, n - nl, X.coff[i], true, false);
-        for (int j = n - nl; j < n; j++) {
-            const int kmax = (v.AT.rowptr[j + 1] - v.AT.rowptr[j] + 31) / 32;
-            t[1].push_back(BlockTile{(int)(X.coff[i] + j), tile_info(1, TILE_LONG, true, false, i), kmax, ~0u, 0, 0, {}});
-            bytes += bytes_of(t[1].back());
-        }
-        cut(v.A, 0, m_eq, X.roff[i], false, false);
-        cut(v.A, m_eq, m, X.roff[i], false, true);
+        if (X.cut[i][0].empty() && X.cut[i][1].empty()) cut_tiles(X, i);
+        for (const auto &list : X.cut[i]) for (const BlockTile &T : list) bytes += T.bytes;
         if (bytes > (int64_t)X.sms * X.blk_smem_max) return;
+    }
+    for (int ph = 0; ph < 2; ph++) {   // the LPs' lists merged, equal tiles in the LPs' order
+        std::vector<size_t> ends{0};
+        for (int i = 0; i < X.k; i++)
+            if (mask[i]) {
+                t[ph].insert(t[ph].end(), X.cut[i][ph].begin(), X.cut[i][ph].end());
+                ends.push_back(t[ph].size());
+            }
+        for (size_t step = 1; step + 1 < ends.size(); step *= 2)
+            for (size_t a = 0; a + step + 1 < ends.size(); a += 2 * step)
+                std::inplace_merge(t[ph].begin() + ends[a], t[ph].begin() + ends[a + step],
+                                   t[ph].begin() + ends[std::min(a + 2 * step, ends.size() - 1)], tile_before);
     }
     const int64_t np = t[1].size(), nd = t[0].size();
     if (np == 0 || nd == 0) return;
@@ -2574,33 +2597,25 @@ static void plan_block(uc_session &X, const std::vector<char> &mask, std::vector
     const bool big = np + nd > (int64_t)kBigTiles * nc * (kMidThreads / 32);
     const int W = (int)std::min<int64_t>((big ? kBigThreads : kMidThreads) / 32, (np + nd + nc - 1) / nc);
     const int64_t S = (int64_t)nc * W;
-    std::vector<std::vector<const BlockTile *>> mine[2];
-    for (int ph = 0; ph < 2; ph++) {
-        mine[ph].resize(S);
-        std::stable_sort(t[ph].begin(), t[ph].end(), [&](const BlockTile &a, const BlockTile &b) {
-            return a.kmax != b.kmax ? a.kmax > b.kmax : bytes_of(a) > bytes_of(b);
-        });
-        for (int64_t i = 0; i < (int64_t)t[ph].size(); i++) mine[ph][ph ? i % S : S - 1 - i % S].push_back(&t[ph][i]);
-    }
-    for (int c = 0; c < nc; c++)
-        for (int w = 0; w < W; w++) {
-            const int64_t slot = (int64_t)w * nc + c;
-            warps.push_back(BlockWarp{(int)tiles.size(), (int)(mine[1][slot].size() + mine[0][slot].size())});
-            for (int ph = 1; ph >= 0; ph--)
-                for (const BlockTile *p : mine[ph][slot]) tiles.push_back(*p);
-        }
     const int head = block_head(X);
     int64_t most = 0, image = 0;
+    tiles.reserve((size_t)(np + nd));
+    warps.reserve((size_t)S);
     for (int c = 0; c < nc; c++) {
         int64_t at = head + (big ? W * kStageBytes : 0);
         for (int w = 0; w < W; w++) {
-            const BlockWarp &wp = warps[(size_t)c * W + w];
-            for (int q = wp.first; q < wp.first + wp.count; q++) {
-                tiles[q].smem = (int)at;
-                tiles[q].img = (int)(image / 16);
-                at += bytes_of(tiles[q]);
-                image += bytes_of(tiles[q]) - kTileOwn;
-            }
+            const int64_t slot = (int64_t)w * nc + c;
+            const size_t first = tiles.size();
+            for (int ph = 1; ph >= 0; ph--)
+                for (int64_t q = ph ? slot : S - 1 - slot; q < (ph ? np : nd); q += S) {
+                    BlockTile T = t[ph][q];
+                    T.smem = (int)at;
+                    T.img = (int)(image / 16);
+                    at += T.bytes;
+                    image += T.bytes - kTileOwn;
+                    tiles.push_back(T);
+                }
+            warps.push_back(BlockWarp{(int)first, (int)(tiles.size() - first)});
         }
         most = std::max(most, at);
     }
@@ -2875,6 +2890,7 @@ static int session_create_as(const PsData *const *Pp, const std::shared_ptr<cons
         X->cta = 128;   // the lanes kernels are built for 128-thread CTAs
     }
     resident = X->block_able;
+    if (!X->block_able) X->cut.clear();
     const int64_t M = X->M, N = X->N, Z = X->Z;
     // CTA tables for every LP (their sizes are the capacities of the device tables)
     std::vector<Seg> sp, sd, se, sa;
