@@ -90,7 +90,7 @@ struct BlockPlan {
     ulonglong2 *xt, *yt;          // x-bar and y, tagged
     unsigned long long *stamp;    // kernel timing: the timed iteration's bounds on CTA 0 (or null)
     int stamp_it, nlps, n_eval, head;   // head: bytes before the warps' staged constants and the tiles
-    unsigned polls;               // a wait's limit
+    unsigned polls;               // a wait's limit (LIMIT instance)
 };
 struct __align__(16) BlockLp { double tau, nsigma; int j, lim, pad[2]; };
 
@@ -110,12 +110,14 @@ __device__ __forceinline__ ulonglong2 ld_tagged(const ulonglong2 *p) {
     return w;
 }
 
-// Every wait ends: after BlockPlan::polls polls (0.3 to 1 us each) stalled is set and the
+// Every wait ends: after kBlockPolls polls (0.3 to 1 us each) stalled is set and the
 // caller leaves.  The CTAs of a cooperative launch start together, once all of them fit
 // beside what other streams run (40 SMs held for 20 ms: all 152 CTAs start within 1 us
 // of one another after that; two such launches of one CTA per SM run one after the
 // other, whatever their streams' priorities), so another kernel delays the launch and
 // never an element; the limit, 10 s at least, only ends what a defect would let hang.
+// A constant: as a kernel argument 0.6 % of an iteration at 30 to 1,441 buses; the LIMIT
+// instance takes it from the plan, for tests of this exit.
 constexpr unsigned kBlockPolls = 1u << 25;
 
 // arrived() + (this lane's entries) . g, in order, N gathers in flight; entry q at
@@ -224,7 +226,7 @@ __global__ void __launch_bounds__(kSmallThreads) k_block_pack(const BlockTile *_
 // (its x is w x-bar + (1 - w) x0, the Halpern step, computed when it is needed
 // next).  The last iteration of the block (or before the limit) writes what the
 // evaluation and the results read.
-template <typename VT, int NT, bool ONE>
+template <typename VT, int NT, bool ONE, bool LIMIT = false>
 __global__ void __launch_bounds__(NT, 1) k_block(const __grid_constant__ BlockPlan P, const __grid_constant__ Bufs b) {
     extern __shared__ __align__(16) unsigned char blk_smem[];
     constexpr int N = NT > kMidThreads ? kBigN : NT > kSmallThreads ? kMidN : kSmallN;
@@ -333,11 +335,11 @@ __global__ void __launch_bounds__(NT, 1) k_block(const __grid_constant__ BlockPl
                 if (primal && it == 0) {
                     acc = plain_dot(arrived(), b.y[0], col, val, add, cnt);
                 } else if (tile_kind(T.y) == TILE_UNIFORM) {
-                    if (kmax == 3) acc = tile_dot<3, true>(gt, want, col, val, add, 3, 3, P.polls, stalled, arrived);
-                    else if (kmax == 2) acc = tile_dot<2, true>(gt, want, col, val, add, 2, 2, P.polls, stalled, arrived);
-                    else if (kmax == 1) acc = tile_dot<1, true>(gt, want, col, val, add, 1, 1, P.polls, stalled, arrived);
-                    else acc = tile_dot<4, true>(gt, want, col, val, add, 4, 4, P.polls, stalled, arrived);
-                } else acc = tile_dot<N, false>(gt, want, col, val, add, kmax, cnt, P.polls, stalled, arrived);
+                    if (kmax == 3) acc = tile_dot<3, true>(gt, want, col, val, add, 3, 3, LIMIT ? P.polls : kBlockPolls, stalled, arrived);
+                    else if (kmax == 2) acc = tile_dot<2, true>(gt, want, col, val, add, 2, 2, LIMIT ? P.polls : kBlockPolls, stalled, arrived);
+                    else if (kmax == 1) acc = tile_dot<1, true>(gt, want, col, val, add, 1, 1, LIMIT ? P.polls : kBlockPolls, stalled, arrived);
+                    else acc = tile_dot<4, true>(gt, want, col, val, add, 4, 4, LIMIT ? P.polls : kBlockPolls, stalled, arrived);
+                } else acc = tile_dot<N, false>(gt, want, col, val, add, kmax, cnt, LIMIT ? P.polls : kBlockPolls, stalled, arrived);
                 if (kmax == 0) acc = arrived();
                 if (stalled) break;
                 if (lng) {
@@ -399,7 +401,7 @@ __global__ void __launch_bounds__(NT, 1) k_block(const __grid_constant__ BlockPl
         }
         if (stalled) break;
     }
-    copy8_wait();   // a wait that ran out may have left a row's constants in flight
+    if (STAGED) copy8_wait();   // a wait that ran out may have left a row's constants in flight
     if (stalled && lane == 0)
         for (int i = 0; i < P.nlps; i++)
             if (b.S[i].status == RUNNING) { b.S[i].status = STALLED; b.status[i] = STALLED; }

@@ -1772,7 +1772,7 @@ struct uc_session {
     int sms = 0, blk_smem_max = 0;          // SMs, shared memory per CTA
     int blk_ctas = 0, blk_threads = 0, blk_smem = 0;
     int64_t blk_image = 0;                  // bytes of the tables' image
-    uc::dev::BlockPlan plan{};
+    uc::dev::BlockPlan plan{.polls = uc::dev::kBlockPolls};
     std::vector<std::array<std::vector<uc::dev::BlockTile>, 2>> cut;   // each LP's tiles, dual and primal (plan_block)
     unsigned long long *h_stamp = nullptr;   // pinned [2][2]: timed iteration's bounds of each graph
     double *h_vec = nullptr;      // pinned: an LP's vectors on their way to the device (update_lp)
@@ -2324,13 +2324,15 @@ static void launch_adaptive_norm(uc_session &X, cudaStream_t s) {
 
 using BlockKernel = void (*)(BlockPlan, Bufs);
 template <typename VT>
-static BlockKernel block_kernel_vt(int threads, bool one) {
+static BlockKernel block_kernel_vt(int threads, bool one, bool limit) {
+    if (limit) return k_block<double, kSmallThreads, true, true>;
     if (threads <= kSmallThreads) return one ? k_block<VT, kSmallThreads, true> : k_block<VT, kSmallThreads, false>;
     if (threads <= kMidThreads) return one ? k_block<VT, kMidThreads, true> : k_block<VT, kMidThreads, false>;
     return one ? k_block<VT, kBigThreads, true> : k_block<VT, kBigThreads, false>;
 }
 static BlockKernel block_kernel(const uc_session &X, int threads) {
-    return X.vb == 32 ? block_kernel_vt<float>(threads, X.k == 1) : block_kernel_vt<double>(threads, X.k == 1);
+    return X.vb == 32 ? block_kernel_vt<float>(threads, X.k == 1, false)
+                      : block_kernel_vt<double>(threads, X.k == 1, X.plan.polls != kBlockPolls);
 }
 static int block_head(const uc_session &X) {
     return (int)(sizeof(BlockLp) * X.k + sizeof(double2) * (X.k == 1 ? X.o.n_eval + 1 : 0));
@@ -3085,7 +3087,6 @@ static int session_create_as(const PsData *const *Pp, const std::shared_ptr<cons
     X->plan.yt = (ulonglong2 *)(D + L.yt);
     X->plan.stamp = o.kernel_timing ? (unsigned long long *)(D + L.stamp) : nullptr;
     X->plan.stamp_it = o.n_eval / 2 - 1;   // its end is the next iteration's start
-    X->plan.polls = kBlockPolls;
     b.S = (Scalars *)(D + L.S);
     b.status = (int *)(D + L.status);
     X->dsp = (const Seg *)(D + L.segs_p); X->dsd = (const Seg *)(D + L.segs_d);
@@ -4098,9 +4099,13 @@ int uc_session_update_lp(uc_session *s, int i, const uc_presolved *ps) {
 }
 
 int uc_session_wait_limit(uc_session *s, unsigned polls) {
-    if (!s) { set_error("uc_session_wait_limit: null session"); return UC_EINVAL; }
+    if (!s || !s->block || s->k != 1 || s->vb != 64 || s->blk_threads > dev::kSmallThreads) {
+        set_error("uc_session_wait_limit: needs a resident session of one small LP with FP64 values");
+        return UC_EINVAL;
+    }
     UC_CUDA(cudaStreamSynchronize(s->s));
     s->plan.polls = polls;
+    UC_CUDA(cudaFuncSetAttribute(dev::block_kernel(*s, s->blk_threads), cudaFuncAttributeMaxDynamicSharedMemorySize, s->blk_smem_max));
     const std::vector<char> tabled = s->tabled;
     return dev::retable(*s, tabled);   // the graphs hold the plan
 }

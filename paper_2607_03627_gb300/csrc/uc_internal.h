@@ -117,8 +117,9 @@ void postsolve(const PsData &ps, const double *xs, const double *ys, std::vector
 
 }  // namespace uc
 
-// Polls after which a wait of the resident block kernel gives up (the LPs still running
-// end UC_ECUDA): for tests of that exit; waits of a working kernel are a few polls long.
+// Polls after which a wait of the resident block kernel gives up (the LP still running ends
+// UC_ECUDA), for tests of that exit: a session of one LP with FP64 values and at most eight
+// warps of tiles per SM.
 extern "C" int uc_session_wait_limit(uc_session *s, unsigned polls);
 
 struct uc_lp {

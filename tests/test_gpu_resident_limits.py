@@ -41,7 +41,7 @@ def _same(B, ra, rb, ps):
 def test_a_wait_that_runs_out_is_an_error_status_and_the_session_goes_on(B):
     # every wait gives up after its second look: the kernel ends, the LP is reported as
     # failed, and with the usual limit the session solves as ever
-    ps = _presolved(B, 6, 300, 24, 36)
+    ps = _presolved(B, 6, 100, 24, 12)
     limit = B.lib.uc_session_wait_limit
     limit.argtypes, limit.restype = [ctypes.c_void_p, ctypes.c_uint], ctypes.c_int
     s = B.Session([ps], tol=0.0, max_iter=640)
