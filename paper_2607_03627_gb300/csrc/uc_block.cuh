@@ -285,7 +285,6 @@ __global__ void __launch_bounds__(NT, 1) k_block(const __grid_constant__ BlockPl
     __syncthreads();
     const int nit = nit_;
     const bool stamps = P.stamp && blockIdx.x == 0 && threadIdx.x == 0;
-    if (stamps) P.stamp[0] = P.stamp[1] = 0;   // of a block that ends before: none
     const unsigned seq = *P.seq;
     bool stalled = false;
 #pragma unroll 1

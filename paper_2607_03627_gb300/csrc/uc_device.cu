@@ -47,7 +47,11 @@ constexpr int kThreads = 256;      // threads per CTA of the row kernels (8 warp
 // Rows handled by one CTA of the evaluation kernel, by the LP's rows + columns
 // (not the session's: a batch evaluates each LP as its single solve does).  Small
 // LPs take one per thread, so that the evaluation, which the FP64 pipe of the few
-// SMs it runs on bounds, spreads over four times the SMs.
+// SMs it runs on bounds, spreads over four times the SMs: up to 608 CTAs, four for each
+// of 152 SMs, before a CTA gets more.  A constant and not the device's SM count: the sums'
+// order, and so the iterates, stay the same on a part of a device.  Evaluation and block
+// start at 256 / 512 / 1024 rows: 47 k rows + columns 30.6 / 31.3 / 40.8 us, 157 k 41.0 /
+// 42.2 / 43.0, 227 k 48.0 / 46.4 / 50.0, 315 k 56.2 / 53.2 / 53.7, 474 k 76.0 / 68.6 / 63.7.
 static int eval_rows(int64_t nm) { return nm <= 256 * 608 ? 256 : nm <= 512 * 608 ? 512 : 1024; }
 constexpr int kSlots = 9;          // reduction slots per candidate
 constexpr int kPart = 2 * kSlots;  // per-block partial record (current, average)
@@ -1775,6 +1779,7 @@ struct uc_session {
     uc::dev::BlockPlan plan{.polls = uc::dev::kBlockPolls};
     std::vector<std::array<std::vector<uc::dev::BlockTile>, 2>> cut;   // each LP's tiles, dual and primal (plan_block)
     unsigned long long *h_stamp = nullptr;   // pinned [2][2]: timed iteration's bounds of each graph
+    unsigned long long last_stamp = 0;       // start of the iteration counted last
     double *h_vec = nullptr;      // pinned: an LP's vectors on their way to the device (update_lp)
     // staged iteration kernels
     bool staged = false;
@@ -3255,7 +3260,10 @@ static int session_run(uc_session &X, int max_replays) {
         if (timing && !done && X.block) {
             // the halves of an iteration overlap: its time is split by their FP64 instructions
             const volatile unsigned long long *t = X.h_stamp + 2 * gi;
-            if (t[0] && t[1] > t[0]) {
+            // a block that ends before the timed iteration leaves an older block's (cleared by
+            // the kernel they cost 0.3 % of an iteration at 300 buses)
+            if (t[0] != X.last_stamp && t[1] > t[0]) {
+                X.last_stamp = t[0];
                 const double ms = (double)(t[1] - t[0]) * 1e-6, p = (double)(X.Z + 4 * X.N), d = (double)(X.Z + 4 * X.M);
                 X.tp_sum += ms * p / (p + d); X.td_sum += ms * d / (p + d); X.timed++;
             }
