@@ -3707,7 +3707,8 @@ __device__ __forceinline__ double kkt_sum_records(const double *rec, int n, int 
 // loads of a row in flight together, FP64 instructions only for the products and
 // sums (bit tests for every comparison, a vote skips a warp's terms that are exact
 // zeros) and about one division per CTA instead of one per row and column.
-// 6,049 buses: 150.9 -> 87.6 us, 30 buses: 26.6 -> 12.4 us per call.
+// 6,049 buses: 150.9 -> 87.4 us, 30 buses: 26.6 -> 12.4 us per call; 84.6 with non-finite
+// reduced costs in a branch of their own (as selects in one line 91.5).
 __global__ void __launch_bounds__(kThreads, kNoAllocCtas) k_kkt_noalloc(uc_device_lp lp, int nbr, int per, const double *__restrict__ x,
                                                           const double *__restrict__ y, double omega, int ticket,
                                                           double *__restrict__ out) {
