@@ -1,6 +1,6 @@
-"""The resident block kernel at its limits: a wait that runs out, blocks too short
-for the timed iteration, what a session uploads,
-sessions that device memory holds only without it."""
+"""The resident block kernel at its limits: a wait that runs out, blocks too short for
+the timed iteration, what a session uploads, sessions that device memory holds only
+without it, tables rebuilt, sessions that fill the SMs side by side."""
 import ctypes
 
 import numpy as np
@@ -143,3 +143,25 @@ def test_tables_are_rebuilt_without_a_pass_over_the_matrices(B):
             [s.result(q) for q in range(3)]
     assert sorted(took)[3] < 0.04 * create
     s.close()
+
+
+def test_sessions_that_each_fill_the_sms_run_side_by_side(B):
+    # three resident sessions with one CTA of 28 warps on every SM, whose registers leave no
+    # room for another's, on streams of both priorities, beside a session on the row kernels: their launches
+    # take turns, and every result is that of the session alone
+    import concurrent.futures as cf
+
+    import torch
+    pss = [_presolved(B, s, 3000, 48, 360) for s in range(2)]
+    kw = dict(tol=0.0, max_iter=1280)
+    alone = [B.uc_solve(ps, **kw)[0] for ps in pss]
+    jobs = [(0, 0, {}), (1, -1, {}), (0, -1, {}), (1, 0, dict(spmv_kernel=1))]
+
+    def one(job):
+        i, priority, more = job
+        with torch.cuda.stream(torch.cuda.Stream(priority=priority)):
+            return [B.uc_solve(pss[i], **kw, **more)[0] for _ in range(3)]
+    with cf.ThreadPoolExecutor(len(jobs)) as ex:
+        for (i, _, _), got in zip(jobs, ex.map(one, jobs)):
+            for r in got:
+                _same(B, alone[i], r, pss[i])
